@@ -899,6 +899,7 @@ struct RowFeed {
   hier_avg* h;
   const void* X_host;
   int G;
+  int64_t cursor0;              // h->cursor at the round's start (the steps advance it)
   int issued_to = 0;            // steps [0, issued_to) have their copies issued
   int chunks = 0;
   std::vector<cudaEvent_t> ev;  // ev[k]: event of step k's chunk
@@ -906,7 +907,7 @@ struct RowFeed {
     const int k0 = issued_to;
     if (k0 >= G) return HA_OK;
     const int k1 = std::min(G, k0 <= 1 ? k0 + 1 : 2 * k0);
-    int64_t r0 = (h->cursor + static_cast<int64_t>(k0) * h->Bstep) % h->N;
+    int64_t r0 = (cursor0 + static_cast<int64_t>(k0) * h->Bstep) % h->N;
     const int64_t rows = static_cast<int64_t>(k1 - k0) * h->Bstep;
     int64_t left = rows < h->N ? rows : h->N;
     if (rows >= h->N) r0 = 0;
@@ -1205,7 +1206,7 @@ int hier_avg_round_host(hier_avg* h, const void* X_host, const int32_t* y_host, 
         (rc = h->cuda(cudaStreamWaitEvent(h->copy_stream, h->round_start, 0), "round_host: wait")) ||
         (rc = copy_labels(h, y_host, h->copy_stream)))
       return rc;
-    RowFeed feed{h, X_host, G};
+    RowFeed feed{h, X_host, G, h->cursor};
     feed.ev.assign(G, nullptr);
     if ((rc = do_round(h, &feed))) return rc;
   }

@@ -635,6 +635,27 @@ def test_round_host_matches_device_round(w, G):
         assert torch.allclose(loss, ha1.losses())
 
 
+# The bound device data set starts empty, so every row that a step reads has to be copied
+# by the round itself: chunk boundaries, the wrap around N, and a second round that
+# starts mid data set.
+@pytest.mark.parametrize("w,G", [(FUSE_THREE, 0), (FUSE_PIECES, 0), (SMALL_BF16.replace(K1=3, N=700), 11),
+                                 (SMALL_BF16.replace(K1=3), 7), (SMALL_FP32, 0), (HOST_ROWS, 0)],
+                         ids=lambda v: getattr(v, "name", str(v)))
+def test_round_host_copies_every_row_it_reads(w, G):
+    ha1, X, y = setup(w)
+    ha2 = HierAvg(w.P, w.S, w.K1, w.K2, w.lr, w.B, w.dims, w.precision)
+    ha2.bind(ha1.params.clone(), torch.zeros_like(X, device="cuda"), torch.zeros_like(y, device="cuda"))
+    for h in (ha1, ha2):
+        h.set_global_steps(G)
+    Xh, yh = X.pin_memory(), y.pin_memory()
+    for _ in range(2):
+        ha1.round()
+        loss = ha2.round_host(Xh, yh)
+        torch.cuda.synchronize()
+        assert torch.equal(ha1.params, ha2.params)
+        assert torch.allclose(loss, ha1.losses())
+
+
 def test_resume_from_saved_step():
     w = SMALL_BF16
     ha1, X, y = setup(w)
