@@ -90,7 +90,7 @@ struct hier_avg {
   std::vector<int> bwd_whole, bwd_np;         // per layer: whole tiles, tail pieces
   bool fused_xent = false;                    // d_L <= 128: CE in the last forward epilogue
   bool w_stream = true;                       // parameters exceed L2: stream W evict-first
-  bool head = false;                          // d_L <= 16: fused last-layer kernel
+  bool head = false;                          // d_L <= 16: fused last-layer kernel (either precision)
   // binding
   bool bound = false;
   int device = 0;
@@ -284,6 +284,7 @@ int plan_layout(hier_avg* h) {
     h->off_dyn = take(16);
   } else {
     for (int l = 0; l <= L; ++l) h->pitch[l] = h->dims[l];
+    h->head = ha::head32_supported(h->dims[L], h->dims[L - 1], static_cast<int>(B));
     for (int l = 0; l < L; ++l) h->off_H[l] = take(P * B * h->dims[l] * 4);
     for (int l = 1; l <= L; ++l) h->off_dZ[l] = take(P * B * h->dims[l] * 4);
   }
@@ -478,6 +479,80 @@ ha::HeadArgs head_args(hier_avg* h, ParamSrc src) {
   }
   a.loss = h->loss();
   return a;
+}
+
+// The rows that layer l reads in the fp32 path: X for the first layer, else H_l.
+ha::F32Rows rows_f32(hier_avg* h, int l) {
+  const int64_t B = h->Bstep, d = h->dims[l];
+  if (l == 0) return {static_cast<const float*>(h->X), h->N * d, h->N, h->cursor % h->N};
+  return {h->wsp<float>(h->off_H[l]), B * d, B, 0};
+}
+
+// The launches of one fp32 step (steps = 1), or of `steps` consecutive steps of a one-layer
+// model whose last layer runs as one kernel (h->head and L = 1).
+int do_step_f32(hier_avg* h, int steps) {
+  const int L = h->L, P = h->P, B = h->Bstep;
+  const int64_t r0 = h->cursor % h->N;
+  cudaStream_t s = h->stream;
+  int rc;
+  const int n_fwd = h->head ? L - 1 : L;
+  for (int l = 0; l < n_fwd; ++l) {
+    const bool last = l + 1 == L;
+    float* outp = last ? h->wsp<float>(h->off_Z) : h->wsp<float>(h->off_H[l + 1]);
+    rc = h->timed(HA_KERNEL_FORWARD, bytes_forward(h, l), flops_gemm(h, l), [&] {
+      return ha::launch_fwd_f32(rows_f32(h, l), h->params + h->woff[l], h->params + h->boff[l], h->ld,
+                                h->dims[l], h->dims[l + 1], B, last ? 0 : 1, outp, P, s);
+    }, "forward");
+    if (rc) return rc;
+  }
+  if (h->head) {
+    const ha::F32Rows hr = rows_f32(h, L - 1);
+    ha::Head32Args a{};
+    a.C = h->dims[L];
+    a.in = h->dims[L - 1];
+    a.B = B;
+    a.ld = h->ld;
+    a.N = h->N;
+    a.row0 = r0;
+    a.steps = steps;
+    a.lr = h->lr;
+    a.W = h->params + h->woff[L - 1];
+    a.bias = h->params + h->boff[L - 1];
+    a.H = hr.base;
+    a.h_stride = hr.stride;
+    a.x_rows = L == 1;
+    a.y = h->y;
+    a.has_dx = L > 1;
+    a.dz_prev = L > 1 ? h->wsp<float>(h->off_dZ[L - 1]) : nullptr;
+    a.loss = h->loss();
+    // W_L read and written once per launch, the batches once
+    const double hb = double(P) * (8.0 * a.C * a.in + steps * 4.0 * B * a.in * (L > 1 ? 2 : 1));
+    rc = h->timed(HA_KERNEL_HEAD, hb, flops_gemm(h, L - 1) * (L > 1 ? 3 : 2) * steps,
+                  [&] { return ha::launch_head_f32(a, P, s); }, "head");
+  } else {
+    rc = h->timed(HA_KERNEL_XENT, double(P) * B * h->dims[L] * 4 * 2, 0.0, [&] {
+      return ha::launch_xent_f32(h->wsp<float>(h->off_Z), h->y, h->N, r0, B, h->dims[L],
+                                 h->wsp<float>(h->off_dZ[L]), h->loss(), P, s);
+    }, "xent");
+  }
+  if (rc) return rc;
+  for (int l = n_fwd - 1; l >= 0; --l) {
+    rc = h->timed(HA_KERNEL_BACKWARD, bytes_backward(h, l), flops_gemm(h, l) * (l > 0 ? 2 : 1), [&] {
+      cudaError_t e = cudaSuccess;
+      if (l > 0) {
+        ++h->launches;                    // dX is its own launch
+        e = ha::launch_dx_f32(h->wsp<float>(h->off_dZ[l + 1]), h->params + h->woff[l], h->ld,
+                              h->wsp<float>(h->off_H[l]), h->dims[l], h->dims[l + 1], B,
+                              h->wsp<float>(h->off_dZ[l]), P, s);
+      }
+      if (e != cudaSuccess) return e;
+      return ha::launch_dw_update_f32(h->wsp<float>(h->off_dZ[l + 1]), rows_f32(h, l),
+                                      h->params + h->woff[l], h->params + h->boff[l], h->ld, h->dims[l],
+                                      h->dims[l + 1], B, h->lr, P, s);
+    }, "backward");
+    if (rc) return rc;
+  }
+  return HA_OK;
 }
 
 // One step.  h1_ready: H_1 of this step was written by the previous step's
@@ -711,42 +786,8 @@ int do_step(hier_avg* h, bool h1_ready = false, bool fuse_next = false, bool* fu
       if (rc) return rc;
     }
   } else {
-    const int d0 = h->dims[0];
-    rc = h->timed(HA_KERNEL_GATHER, double(P) * B * d0 * 4 * 2, 0.0, [&] {
-      return ha::launch_gather_f32(static_cast<const float*>(h->X), h->N, d0, B, h->cursor % h->N, P,
-                                   h->wsp<float>(h->off_H[0]), s);
-    }, "gather");
+    rc = do_step_f32(h, 1);
     if (rc) return rc;
-    for (int l = 0; l < L; ++l) {
-      const bool last = l + 1 == L;
-      float* outp = last ? h->wsp<float>(h->off_Z) : h->wsp<float>(h->off_H[l + 1]);
-      rc = h->timed(HA_KERNEL_FORWARD, bytes_forward(h, l), flops_gemm(h, l), [&] {
-        return ha::launch_fwd_f32(h->wsp<float>(h->off_H[l]), h->params + h->woff[l],
-                                  h->params + h->boff[l], h->ld, h->dims[l], h->dims[l + 1], B,
-                                  last ? 0 : 1, outp, P, s);
-      }, "forward");
-      if (rc) return rc;
-    }
-    rc = h->timed(HA_KERNEL_XENT, double(P) * B * h->dims[L] * 4 * 2, 0.0, [&] {
-      return ha::launch_xent_f32(h->wsp<float>(h->off_Z), h->y, h->N, h->cursor % h->N, B, h->dims[L],
-                                 h->wsp<float>(h->off_dZ[L]), h->loss(), P, s);
-    }, "xent");
-    if (rc) return rc;
-    for (int l = L - 1; l >= 0; --l) {
-      rc = h->timed(HA_KERNEL_BACKWARD, bytes_backward(h, l), flops_gemm(h, l) * (l > 0 ? 2 : 1), [&] {
-        cudaError_t e = cudaSuccess;
-        if (l > 0) ++h->launches;   // dX is its own launch
-        if (l > 0)
-          e = ha::launch_dx_f32(h->wsp<float>(h->off_dZ[l + 1]), h->params + h->woff[l], h->ld,
-                                h->wsp<float>(h->off_H[l]), h->dims[l], h->dims[l + 1], B,
-                                h->wsp<float>(h->off_dZ[l]), P, s);
-        if (e != cudaSuccess) return e;
-        return ha::launch_dw_update_f32(h->wsp<float>(h->off_dZ[l + 1]), h->wsp<float>(h->off_H[l]),
-                                        h->params + h->woff[l], h->params + h->boff[l], h->ld,
-                                        h->dims[l], h->dims[l + 1], B, h->lr, P, s);
-      }, "backward");
-      if (rc) return rc;
-    }
   }
   ++h->t;
   h->cursor += B;
@@ -946,8 +987,23 @@ int do_round(hier_avg* h, RowFeed* feed = nullptr) {
   const int G = round_steps(h);
   const bool compact = h->m_ok;
   bool h1_ready = false;
+  // fp32 softmax regression (one layer of at most 16 classes): the steps up to the next
+  // average run in one launch.
+  const bool multi = h->prec != HA_PREC_BF16 && h->head && h->L == 1;
   for (int r = 1; r <= G; ++r) {
     const int k = r - 1;
+    if (multi) {
+      const int n = std::min(h->K1 - k % h->K1, G - k);
+      if ((rc = do_step_f32(h, n))) return rc;
+      h->t += n;
+      h->cursor += static_cast<int64_t>(n) * h->Bstep;
+      r += n - 1;
+      if (r % h->K1 == 0) {
+        if (r == G) return do_local_global(h);
+        if ((rc = do_local(h))) return rc;
+      }
+      continue;
+    }
     if (feed && (k == 0 || (k & (k + 1)) == 0)) {
       const int need = k == 0 ? 0 : std::min(2 * k + 1, G - 1);
       if ((rc = feed->ensure(std::max(need, std::min(1, G - 1))))) return rc;
@@ -1136,6 +1192,8 @@ int hier_avg_bind(hier_avg* h, float* params_dev, void* workspace_dev, int64_t w
     if ((rc = h->cuda(ha::tc_configure(), "bind: kernel attributes"))) return rc;
     if ((rc = h->cuda(ha::head_configure(), "bind: kernel attributes"))) return rc;
     if ((rc = build_maps(h))) return rc;
+  } else if ((rc = h->cuda(ha::fp32_configure(), "bind: kernel attributes"))) {
+    return rc;
   }
   h->bound = true;
   return HA_OK;
@@ -1464,6 +1522,8 @@ extern "C" int hier_avg_step_static(hier_avg* h, float* params_dev, const void* 
     if ((rc = h->cuda(ha::tc_configure(), "step_static: kernel attributes"))) return rc;
     if ((rc = h->cuda(ha::head_configure(), "step_static: kernel attributes"))) return rc;
     if ((rc = build_maps(h))) return rc;
+  } else if ((rc = h->cuda(ha::fp32_configure(), "step_static: kernel attributes"))) {
+    return rc;
   }
   h->bound = true;
   return do_step(h);

@@ -215,17 +215,39 @@ cudaError_t launch_head(const HeadArgs& a, int P, cudaStream_t s);
 
 // ----------------------------------------------------------------- fp32 CUDA-core step
 // Buffers: H_l [P][B][d_l] fp32, Z_L [P][B][d_L], dZ_l [P][B][d_l] fp32.
-cudaError_t launch_gather_f32(const float* X, int64_t N, int d0, int B, int64_t row0, int P,
-                              float* H0, cudaStream_t s);
-cudaError_t launch_fwd_f32(const float* H, const float* W, const float* bias, int64_t ld,
-                           int in, int out, int B, int relu, float* out_act, int P,
-                           cudaStream_t s);
+// A layer's input rows: learner j's batch row b is row (row0 + b) mod N of base + j * stride
+// (X itself for the first layer, H_l with N = B and row0 = 0 for the others).
+struct F32Rows {
+  const float* base;
+  int64_t stride, N, row0;
+};
+// The last layer in one launch, for at most 16 classes and 64 samples (head32_supported).
+struct Head32Args {
+  int C, in, B;
+  int64_t ld, N, row0;        // first row of the launch's first batch in each learner's data
+  int steps;                  // local steps in this launch (1 unless x_rows)
+  float lr;
+  float* W;                   // learner 0's W_L [C][in]
+  float* bias;                // learner 0's b_L
+  const float* H;             // H_{L-1} [P][B][in], or X [P][N][in] when x_rows
+  int64_t h_stride;           // floats from one learner's rows to the next's
+  int x_rows;
+  const int32_t* y;
+  int has_dx;                 // write dZ_{L-1}
+  float* dz_prev;             // [P][B][in]
+  float* loss;                // [P]
+  int bufs, vec;              // set by the launcher: batch buffers, 16-byte rows
+};
+cudaError_t fp32_configure();   // raises the dynamic shared-memory limits once
+bool head32_supported(int C, int in, int B);
+cudaError_t launch_head_f32(const Head32Args& a, int P, cudaStream_t s);
+cudaError_t launch_fwd_f32(const F32Rows& h, const float* W, const float* bias, int64_t ld, int in,
+                           int out, int B, int relu, float* out_act, int P, cudaStream_t s);
 cudaError_t launch_xent_f32(const float* Z, const int32_t* y, int64_t N, int64_t row0, int B,
                             int C, float* dZ, float* loss, int P, cudaStream_t s);
-cudaError_t launch_dx_f32(const float* dZ, const float* W, int64_t ld, const float* Hprev,
-                          int in, int out, int B, float* dZprev, int P, cudaStream_t s);
-cudaError_t launch_dw_update_f32(const float* dZ, const float* H, float* W, float* bias,
-                                 int64_t ld, int in, int out, int B, float lr, int P,
-                                 cudaStream_t s);
+cudaError_t launch_dx_f32(const float* dZ, const float* W, int64_t ld, const float* Hprev, int in,
+                          int out, int B, float* dZprev, int P, cudaStream_t s);
+cudaError_t launch_dw_update_f32(const float* dZ, const F32Rows& h, float* W, float* bias, int64_t ld,
+                                 int in, int out, int B, float lr, int P, cudaStream_t s);
 
 }  // namespace ha

@@ -76,6 +76,15 @@ __device__ __forceinline__ void cluster_sync_all() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;"
                ::: "memory");
 }
+// The float at the same shared-memory offset in CTA `rank` of this cluster.
+__device__ __forceinline__ float ld_cluster_f1(const float* p, int rank) {
+  const uint32_t la = static_cast<uint32_t>(__cvta_generic_to_shared(p));
+  uint32_t ra;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(la), "r"(rank));
+  float v;
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(ra) : "memory");
+  return v;
+}
 // The four floats at the same shared-memory offset in CTA `rank` of this cluster.
 __device__ __forceinline__ float4 ld_cluster_f4(const float* p, int rank) {
   const uint32_t la = static_cast<uint32_t>(__cvta_generic_to_shared(p));

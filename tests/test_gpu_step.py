@@ -668,3 +668,50 @@ def test_resume_from_saved_step():
     ha2.round()
     torch.cuda.synchronize()
     assert torch.equal(ha1.params, ha2.params)
+
+
+# fp32 kernels at the edges of their tiles: tiles of 8, 16, 32 and 64 samples with one
+# sample missing or too many; widths that are no multiple of 4 (4-byte copies) or end inside
+# a 64-wide chunk; a reduction split over a cluster of 8 (one learner, 2048 inputs); the
+# small last layer at its limits (16 classes, 64 samples, slices of 64 features, one odd
+# slice) and just past them (17 classes, 65 samples, more than 8 x 1024 features).
+def _fp32(dims, P, S, B, **kw):
+    return configs.Workload("fp32_" + "-".join(map(str, dims)) + f"_P{P}_B{B}", P=P, S=S, K1=kw.get("K1", 2),
+                            K2=2, rounds=1, dims=dims, precision="fp32", N=kw.get("N", 3 * B + 1), B=B,
+                            lr=0.05, sigma_mu=0.1, init="he")
+
+
+FP32_CASES = [_fp32((64, 64, 17), 4, 2, 8), _fp32((130, 65, 40), 3, 1, 9), _fp32((260, 132, 128, 300), 2, 2, 33),
+              _fp32((100, 36, 10), 2, 1, 65), _fp32((2048, 64, 10), 1, 1, 32), _fp32((96, 72, 40), 2, 1, 130),
+              _fp32((3072, 10), 2, 2, 64), _fp32((512, 16), 3, 1, 1), _fp32((37, 10), 4, 4, 17),
+              _fp32((70, 5), 2, 2, 3), _fp32((8200, 10), 1, 1, 2), _fp32((516, 61, 16), 2, 1, 16),
+              _fp32((516, 61, 16), 2, 1, 31)]
+
+
+@pytest.mark.parametrize("w", FP32_CASES, ids=lambda w: w.name)
+def test_fp32_step_at_tile_edges(w):
+    test_one_step_from_distinct_learners(w)
+
+
+# One-layer fp32 models run the steps between two averages in one launch: the bits of the
+# single steps, with batches that wrap around the data set, a last block shorter than K1,
+# one batch buffer instead of two (64 samples of 3072 features), and 4-byte copies.
+@pytest.mark.parametrize("w,G", [(configs.SOFTMAX_P4, 0), (_fp32((3072, 10), 4, 2, 64), 5),
+                                 (_fp32((37, 13), 6, 3, 5, K1=3, N=11), 7)],
+                         ids=lambda v: getattr(v, "name", str(v)))
+def test_fp32_steps_in_one_launch(w, G):
+    ha1, X, y = setup(w, perturb=(0.01, 0.01))
+    ha2, _, _ = setup(w, perturb=(0.01, 0.01))
+    ha1.set_global_steps(G)
+    for _ in range(2):
+        ha1.round()
+        n = G or w.K1 * w.K2
+        for r in range(1, n + 1):
+            ha2.step()
+            if r % w.K1 == 0:
+                ha2.local_average()
+        ha2.global_average()
+    torch.cuda.synchronize()
+    assert ha1.get_step() == ha2.get_step() == 2 * n
+    assert torch.equal(ha1.params.view(torch.int32), ha2.params.view(torch.int32))
+    assert torch.equal(ha1.losses(), ha2.losses())
