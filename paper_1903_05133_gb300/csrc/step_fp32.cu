@@ -11,9 +11,9 @@
 // The first layer reads its batch rows straight from X (no gather).  Rows whose length is a
 // multiple of four floats move as 16-byte cp.async copies, others as 4-byte ones.
 // Rounds against 16 x 16-tile kernels with one output per thread and a serial reduction
-// (seven launches per step of a two-layer net): 3072-10 (P = 4, B = 16, 4 steps) 350 -> 30 us,
-// 100-37-10 (P = 4, B = 7, 4 steps) 127 -> 54 us, 3072-512-10 (P = 16, B = 32, 8 steps)
-// 4965 -> 1077 us; error against 64 bits the same or smaller (5e-8 at 3072-10, was 1.2e-7).
+// (seven launches per step of a two-layer net): 3072-10 (P = 4, B = 16, 4 steps) 350 -> 29 us,
+// 100-37-10 (P = 4, B = 7, 4 steps) 127 -> 50 us, 3072-512-10 (P = 16, B = 32, 8 steps)
+// 4965 -> 990 us; error against 64 bits the same or smaller (5e-8 at 3072-10, was 1.2e-7).
 #include <cstdint>
 #include <cuda_runtime.h>
 
@@ -39,29 +39,51 @@ __device__ __forceinline__ void cp_async_wait() {
   asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
-// Columns [k0, k0 + W) of `rows` rows into dst (row stride `pitch` floats) by 256 threads;
-// row(r) is the address of row r (nullptr: zeros), columns from kmax on are zeros.  vec:
-// every row starts on 16 bytes and kmax is a multiple of 4.
-template <int W, class Row>
-__device__ __forceinline__ void load_rows(float* dst, int pitch, int rows, int k0, int kmax, bool vec,
+// r mod N for a row index r >= 0 of a batch: almost always below N, or one turn past it (a
+// 64-bit modulo is ~100 instructions).
+__device__ __forceinline__ int64_t wrap_row(int64_t r, int64_t N) {
+  if (r < N) return r;
+  return r - N < N ? r - N : r % N;
+}
+
+// Columns [k0, k0 + W) of rows [0, R) into dst (row pitch `pitch` floats) by 256 threads;
+// row(r) is the address of row r's column 0 (nullptr: zeros), columns from kmax on are
+// zeros.  vec: every row starts on 16 bytes and kmax is a multiple of 4.
+template <int W, int R, class Row>
+__device__ __forceinline__ void load_rows(float* dst, int pitch, int k0, int kmax, bool vec,
                                           const float* any, int t, Row row) {
   if (vec) {
     constexpr int Q = W / 4;
     const int q = t % Q, k = k0 + 4 * q;
-    for (int r = t / Q; r < rows; r += 256 / Q) {
+    const bool kin = k < kmax;
+#pragma unroll
+    for (int i = 0; i < (R * Q + 255) / 256; ++i) {
+      const int r = t / Q + i * (256 / Q);
+      if (R * Q % 256 != 0 && r >= R) break;
       const float* p = row(r);
-      const bool ok = p != nullptr && k < kmax;
+      const bool ok = p != nullptr && kin;
       cp_async16(dst + r * pitch + 4 * q, ok ? p + k : any, ok);
     }
   } else {
     const int q = t % W, k = k0 + q;
-    for (int r = t / W; r < rows; r += 256 / W) {
+    const bool kin = k < kmax;
+#pragma unroll 4
+    for (int r = t / W; r < R; r += 256 / W) {
       const float* p = row(r);
-      const bool ok = p != nullptr && k < kmax;
+      const bool ok = p != nullptr && kin;
       cp_async4(dst + r * pitch + q, ok ? p + k : any, ok);
     }
   }
 }
+// Weight rows r0 + r < rmax of a row-major matrix W [rmax][in].
+struct WRows {
+  const float* p;     // row r0
+  int64_t in;
+  int rows;           // rmax - r0
+  __device__ __forceinline__ const float* operator()(int r) const {
+    return r < rows ? p + r * in : nullptr;
+  }
+};
 
 // ------------------------------------------------------------------ forward and dX tiles
 // Both contract a [samples x K] operand (H, or dZ) with the weights into a tile of BM
@@ -72,14 +94,14 @@ __device__ __forceinline__ void load_rows(float* dst, int pitch, int rows, int k
 // bandwidth at the FFMA rate).  With few tiles a cluster of up to 8 CTAs shares a tile's
 // chunks.  The partials meet in shared memory and then through distributed shared memory,
 // added in a fixed order (warp, then CTA rank).  Operands arrive by cp.async, three chunks
-// deep.  The forward of 3072 -> 512 (P = 16, B = 32) takes 62 us, 26 TFLOP/s.
+// deep.  The forward of 3072 -> 512 (P = 16, B = 32) takes 58 us, 28 TFLOP/s.
 constexpr int kThreads = 256;
 constexpr int kBN = 64;                 // columns of a tile
 constexpr int kKC = 64;                 // reduction chunk
 constexpr int kKP = kKC + 4;            // row pitch: consecutive rows on distinct bank groups
 constexpr int kRP = kBN + 8;            // row pitch of the partials
 constexpr int kStages = 3;
-constexpr int kTargetCtas = 2 * 152;    // two CTAs per SM
+constexpr int kSms = 152;               // of a GB300
 
 __host__ __device__ constexpr int tile_stage_floats(int BM) { return (BM + kBN) * kKP; }
 __host__ __device__ constexpr int tile_smem(int BM) { return kStages * tile_stage_floats(BM) * 4; }
@@ -120,7 +142,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_tile_f32(const TileArgs a, int 
   const int nk = (K + kKC - 1) / kKC;
   const int c_lo = rank * nk / split, c_hi = (rank + 1) * nk / split;
   if (t < BM)
-    arow[t] = b0 + t < a.B ? a.act + j * a.act_stride + (a.row0 + b0 + t) % a.N * K : nullptr;
+    arow[t] = b0 + t < a.B ? a.act + j * a.act_stride + wrap_row(a.row0 + b0 + t, a.N) * K : nullptr;
   const float* W = a.W + j * a.ld;
   __syncthreads();
   grid_dep_wait();
@@ -128,15 +150,13 @@ __global__ void __launch_bounds__(kThreads, 2) k_tile_f32(const TileArgs a, int 
   auto load = [&](int c, int s) {
     float* as = sm + s * tile_stage_floats(BM);
     float* ws = as + BM * kKP;
-    load_rows<kKC>(as, kKP, BM, c * kKC, K, a.vec_act, a.W, t, [&](int r) { return arow[r]; });
+    load_rows<kKC, BM>(as, kKP, c * kKC, K, a.vec_act, a.W, t, [&](int r) { return arow[r]; });
     if constexpr (kDx)        // rows o of the chunk, columns i of the tile
-      load_rows<kBN>(ws, kBN, kKC, n0, a.in, a.vec_w, a.W, t, [&](int r) {
-        return c * kKC + r < a.out ? W + static_cast<int64_t>(c * kKC + r) * a.in : nullptr;
-      });
+      load_rows<kBN, kKC>(ws, kBN, n0, a.in, a.vec_w, a.W, t,
+                          WRows{W + static_cast<int64_t>(c) * kKC * a.in, a.in, a.out - c * kKC});
     else                      // rows o of the tile, columns k of the chunk
-      load_rows<kKC>(ws, kKP, kBN, c * kKC, a.in, a.vec_w, a.W, t, [&](int r) {
-        return n0 + r < a.out ? W + static_cast<int64_t>(n0 + r) * a.in : nullptr;
-      });
+      load_rows<kKC, kBN>(ws, kKP, c * kKC, a.in, a.vec_w, a.W, t,
+                          WRows{W + static_cast<int64_t>(n0) * a.in, a.in, a.out - n0});
   };
   const int ks = warp % KS, wm = warp / KS, ly = lane >> 3, lx = lane & 7;
   float acc[TM][8];
@@ -273,7 +293,8 @@ __global__ void __launch_bounds__(kThreads, 2) k_tile_f32(const TileArgs a, int 
 // chain per weight) and, in the first input tile, b_l -= lr * sum_b dZ.  CTA = 64 outputs x
 // 128 inputs, thread = 8 x 8 of them; the weights are loaded into registers before the
 // batch arrives, so their latency hides behind the products.  Samples go in chunks of 32
-// through two cp.async stages.  3072 -> 512 (P = 16, B = 32): 61 us, 3.3 TB/s, 26 TFLOP/s.
+// through two cp.async stages.  3072 -> 512 (P = 16, B = 32): 57 us, 3.5 TB/s, 28 TFLOP/s
+// (61 us with a 64-bit modulo per batch row).
 constexpr int kDwThreads = 128;
 constexpr int kDwO = 64, kDwI = 128, kDwB = 32;
 constexpr int kDwStage = kDwB * (kDwO + kDwI);
@@ -309,7 +330,7 @@ __global__ void __launch_bounds__(kDwThreads, 3) k_dw_f32(const DwArgs a) {
       const int b = c * kDwB + r;
       const bool live = b < a.B;
       const float* z = a.dZ + (j * a.B + (live ? b : 0)) * a.out;
-      const float* h = Hj + (a.row0 + (live ? b : 0)) % a.N * a.in;
+      const float* h = Hj + wrap_row(a.row0 + (live ? b : 0), a.N) * a.in;
       if (a.vec_z) {
         if (lane < 16) {
           const bool ok = live && o0 + 4 * lane < a.out;
@@ -519,14 +540,14 @@ __global__ void __launch_bounds__(kThreads) k_head_f32(const Head32Args a) {
       for (int idx = t; idx < B * nq; idx += kThreads) {
         const int b = idx / nq, q = idx - b * nq;
         const bool ok = 4 * q < kc;
-        const float* p = hj + (a.x_rows ? (r0 + b) % N : b) * in + k0 + 4 * q;
+        const float* p = hj + (a.x_rows ? wrap_row(r0 + b, N) : b) * in + k0 + 4 * q;
         cp_async16(hs + b * F + 4 * q, ok ? p : W, ok);
       }
     } else {
       for (int idx = t; idx < B * F; idx += kThreads) {
         const int b = idx / F, f = idx - b * F;
         const bool ok = f < kc;
-        const float* p = hj + (a.x_rows ? (r0 + b) % N : b) * in + k0 + f;
+        const float* p = hj + (a.x_rows ? wrap_row(r0 + b, N) : b) * in + k0 + f;
         cp_async4(hs + b * F + f, ok ? p : W, ok);
       }
     }
@@ -721,13 +742,24 @@ __global__ void __launch_bounds__(kThreads) k_head_f32(const Head32Args a) {
 
 bool aligned16(const void* p) { return reinterpret_cast<uintptr_t>(p) % 16 == 0; }
 
-// CTAs of a cluster that share a tile's reduction: as many (a power of two up to 8) as
-// bring the grid to about two CTAs per SM while each keeps at least two chunks.
+// CTAs of a cluster that share a tile's reduction (a power of two up to 8, at least two
+// chunks each): the least work on the fullest SM, in chunks, with four chunks' worth of
+// start and reduction per CTA, and a fifth on top where every SM holds one CTA at most
+// (nothing covers its waits).  3072 -> 512 (P = 16, B = 32: 128 tiles of 48 chunks), split
+// 1, 2, 4, 8: 63.5, 58.3, 63.2, 68.2 us.
 int tile_split(int64_t tiles, int K) {
-  const int nk = (K + kKC - 1) / kKC;
-  int s = 1;
-  while (s < 8 && tiles * s < kTargetCtas && nk >= 4 * s) s *= 2;
-  return s;
+  const int64_t nk = (K + kKC - 1) / kKC;
+  int best = 1;
+  int64_t cost = 0;
+  for (int s = 1; s <= 8 && (s == 1 || nk >= 2 * s); s *= 2) {
+    const int64_t per_sm = (tiles * s + kSms - 1) / kSms;
+    const int64_t c = per_sm * ((nk + s - 1) / s + 4) * (per_sm == 1 ? 6 : 5);
+    if (s == 1 || c < cost) {
+      cost = c;
+      best = s;
+    }
+  }
+  return best;
 }
 
 template <int BM, bool kDx>
