@@ -182,89 +182,213 @@ __global__ void __launch_bounds__(256) k_local_global_pow2_split(const float4* s
   if (valid) store_rows(w + c + static_cast<int64_t>(g0) * S * ld_v, ld_v, G2 * S, part[threadIdx.x]);
 }
 
-// Generic path: any n (also non-powers of two) and scalar columns.  The binary
-// counter lives in a small local array; after n pushes its pending partials are
-// the set bits of n, folded from the smallest upward.
-template <class V>
-__device__ V tree_any(const V* __restrict__ p, int64_t ld_v, int n) {
-  V stack[32];
-  for (int i = 0; i < n; ++i) {
-    V x = p[static_cast<int64_t>(i) * ld_v];
+// Generic path: any number of rows, any alignment, any row length.  A thread owns four
+// columns, which an access policy maps to memory: Quad for rows that start on 16 bytes (four
+// neighbours, one 128-bit access; the row's last quad may be partial), Spread for all others
+// (columns 256 apart, so that each of the four 32-bit accesses of a warp is contiguous).
+// Everything lives in registers: the tree over n rows is the tree over the complete block of
+// each set bit of n, highest bit first, folded from the smallest block upward (the binary
+// counter's pending partials), and each block is unrolled with its loads in flight.  (One
+// column per thread with the counter in a local array had been bound by the latency of its
+// serial loads and stack.  Unaligned rows, L2 holding the matrix: P = 12, S = 6, D = 1000003
+// local 23.4 -> 12.5 us, local + global 34.0 -> 17.0 us (5.6 TB/s); P = 48, S = 8, D = 8000001
+// from HBM: local 905 -> 459 us (6.7 TB/s), global 880 -> 622, local + global 1067 -> 699.)
+struct Quad {
+  using V = float4;
+  static constexpr int kCols = 4;
+  int64_t c;
+  int live;
+  __device__ __forceinline__ explicit Quad(int64_t cols) {
+    c = (static_cast<int64_t>(blockIdx.x) * 256 + threadIdx.x) * 4;
+    live = cols - c >= 4 ? 4 : cols > c ? static_cast<int>(cols - c) : 0;
+  }
+  __device__ __forceinline__ float4 load(const float* row) const {
+    if (live == 4) return *reinterpret_cast<const float4*>(row + c);
+    return make_float4(row[c], live > 1 ? row[c + 1] : 0.f, live > 2 ? row[c + 2] : 0.f, 0.f);
+  }
+  __device__ __forceinline__ void store(float* row, float4 v) const {
+    if (live == 4) {
+      *reinterpret_cast<float4*>(row + c) = v;
+      return;
+    }
+    row[c] = v.x;
+    if (live > 1) row[c + 1] = v.y;
+    if (live > 2) row[c + 2] = v.z;
+  }
+};
+struct Spread {
+  using V = float4;
+  static constexpr int kCols = 4;
+  int64_t c;
+  int live;
+  __device__ __forceinline__ explicit Spread(int64_t cols) {
+    c = static_cast<int64_t>(blockIdx.x) * 1024 + threadIdx.x;
+    const int64_t left = cols - c;
+    live = left <= 0 ? 0 : left > 768 ? 4 : left > 512 ? 3 : left > 256 ? 2 : 1;
+  }
+  __device__ __forceinline__ float4 load(const float* row) const {
+    const float* p = row + c;
+    return make_float4(p[0], live > 1 ? p[256] : 0.f, live > 2 ? p[512] : 0.f, live > 3 ? p[768] : 0.f);
+  }
+  __device__ __forceinline__ void store(float* row, float4 v) const {
+    float* p = row + c;
+    p[0] = v.x;
+    if (live > 1) p[256] = v.y;
+    if (live > 2) p[512] = v.z;
+    if (live > 3) p[768] = v.w;
+  }
+};
+
+// One column per thread, for rows so short that four would leave SMs without a CTA.
+struct Single {
+  using V = float;
+  static constexpr int kCols = 1;
+  int64_t c;
+  int live;
+  __device__ __forceinline__ explicit Single(int64_t cols) {
+    c = static_cast<int64_t>(blockIdx.x) * 256 + threadIdx.x;
+    live = c < cols;
+  }
+  __device__ __forceinline__ float load(const float* row) const { return row[c]; }
+  __device__ __forceinline__ void store(float* row, float v) const { row[c] = v; }
+};
+
+// Tree over the 2^LOG rows from p on.
+template <int LOG, class A>
+__device__ __forceinline__ typename A::V tree_block(const A& a, const float* p, int64_t ld) {
+  typename A::V stack[LOG + 1];
+#pragma unroll
+  for (int i = 0; i < (1 << LOG); ++i) {
+    typename A::V x = a.load(p + i * ld);
     int l = 0;
-    while ((i >> l) & 1) {
+#pragma unroll
+    for (; l < LOG; ++l) {
+      if (((i >> l) & 1) == 0) break;
       x = vadd(stack[l], x);
-      ++l;
     }
     stack[l] = x;
   }
-  V acc{};
-  bool have = false;
-  for (int l = 0; l < 32; ++l) {
-    if ((n >> l) & 1) {
-      acc = have ? vadd(stack[l], acc) : stack[l];
-      have = true;
+  return stack[LOG];
+}
+
+// The binary counter over values pushed in order, with blocks of 2^level values that are
+// equal or already summed pushed at once (idx: the block's first value, a multiple of
+// 2^level).  The levels are unrolled and uniform over the CTA, so the partials stay in
+// registers.
+template <class V, int LEVELS>
+struct Counter {
+  V st[LEVELS];
+  __device__ __forceinline__ void push(int idx, int level, V x) {
+    bool open = true;
+#pragma unroll
+    for (int l = 0; l < LEVELS; ++l) {
+      if (l < level || !open) continue;
+      if ((idx >> l) & 1) {
+        x = vadd(st[l], x);
+      } else {
+        st[l] = x;
+        open = false;
+      }
     }
+  }
+  // The pending partials of n values folded from the smallest upward, after `acc` (the sum of
+  // smaller blocks that follow them) if have.
+  __device__ __forceinline__ V total(int n, V acc, bool have) const {
+#pragma unroll
+    for (int l = 0; l < LEVELS; ++l)
+      if ((n >> l) & 1) {
+        acc = have ? vadd(st[l], acc) : st[l];
+        have = true;
+      }
+    return acc;
+  }
+};
+
+// Tree over n < 2^BITS rows from p on.  The block of bit l is rows [n with bits 0 .. l
+// cleared, + 2^l).  Above the last n mod 16 rows, kUnroll has one unrolled block per bit (45
+// registers, as many loads in flight as the power-of-two kernels, long code), otherwise
+// blocks of 16 go through a counter.
+template <int BITS, bool kUnroll, class A>
+__device__ __forceinline__ typename A::V tree_rows(const A& a, const float* p, int64_t ld, int n) {
+  typename A::V acc{};
+  bool have = false;
+  auto fold = [&](typename A::V x) {
+    acc = have ? vadd(x, acc) : x;
+    have = true;
+  };
+  auto block = [&](int l) { return p + static_cast<int64_t>((n >> l >> 1) << l << 1) * ld; };
+  if (n & 1) fold(tree_block<0>(a, block(0), ld));
+  if (n & 2) fold(tree_block<1>(a, block(1), ld));
+  if (n & 4) fold(tree_block<2>(a, block(2), ld));
+  if (n & 8) fold(tree_block<3>(a, block(3), ld));
+  if constexpr (BITS > 4 && kUnroll) {
+    static_assert(BITS == 8, "one block per bit");
+    if (n & 16) fold(tree_block<4>(a, block(4), ld));
+    if (n & 32) fold(tree_block<5>(a, block(5), ld));
+    if (n & 64) fold(tree_block<6>(a, block(6), ld));
+    if (n & 128) fold(tree_block<7>(a, block(7), ld));
+  } else if constexpr (BITS > 4) {
+    Counter<typename A::V, BITS - 4> cnt;
+#pragma unroll 1
+    for (int i = 0; i < (n >> 4); ++i) {
+      const float* q = p + static_cast<int64_t>(16 * i) * ld;
+      const typename A::V x = tree_block<3>(a, q, ld);
+      cnt.push(i, 0, vadd(x, tree_block<3>(a, q + 8 * ld, ld)));
+    }
+    acc = cnt.total(n >> 4, acc, have);
   }
   return acc;
 }
 
-template <class V>
-__global__ void __launch_bounds__(256) k_mean_any(V* __restrict__ w, int64_t ld_v,
-                                                  int64_t cols_v, int n) {
+// Sums of groups of n rows of src divided by div: written to all n rows of the group (dst =
+// src's matrix, row stride ld), or, kTo, once, to row g of dst (row stride dst_ld).
+template <class A, int BITS, bool kTo>
+__global__ void __launch_bounds__(256) k_mean_any(const float* src, int64_t ld, int64_t cols, int n,
+                                                  float div, float* dst, int64_t dst_ld) {
   grid_dep_wait();
-  const int64_t c = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (c >= cols_v) return;
-  V* p = w + static_cast<int64_t>(blockIdx.y) * n * ld_v + c;
-  const V m = vdiv(tree_any(p, ld_v, n), static_cast<float>(n));
-  store_rows(p, ld_v, n, m);
+  const A a(cols);
+  if (a.live == 0) return;
+  const int64_t row0 = static_cast<int64_t>(blockIdx.y) * n;
+  const typename A::V m = vdiv(tree_rows<BITS, A::kCols == 4 && !kTo>(a, src + row0 * ld, ld, n), div);
+  if constexpr (kTo) {
+    a.store(dst + static_cast<int64_t>(blockIdx.y) * dst_ld, m);
+  } else {
+#pragma unroll 8
+    for (int i = 0; i < n; ++i) a.store(dst + (row0 + i) * ld, m);
+  }
 }
 
-template <class V>
-__global__ void __launch_bounds__(256) k_mean_any_to(const V* __restrict__ w, int64_t ld_v,
-                                                     int64_t cols_v, int n, float div,
-                                                     V* __restrict__ out, int64_t out_ld_v) {
-  grid_dep_wait();
-  const int64_t c = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (c >= cols_v) return;
-  const V* p = w + static_cast<int64_t>(blockIdx.y) * n * ld_v + c;
-  out[static_cast<int64_t>(blockIdx.y) * out_ld_v + c] = vdiv(tree_any(p, ld_v, n), div);
-}
-
-// (src, src_ld_v, n: as in k_local_global_pow2, n = S / Q source rows per cluster.)
-template <class V>
-__global__ void __launch_bounds__(256) k_local_global_any(const V* src, int64_t src_ld_v, int n,
-                                                          V* w, int64_t ld_v, int64_t cols_v, int S,
+// (src, src_ld, n: as in k_local_global_pow2, n = S / Q source rows per cluster.)  The global
+// tree runs over S copies of each cluster mean; a complete block of 2^l copies is the mean
+// added to itself l times, so a cluster's run is pushed as its maximal aligned blocks.
+// (BITS: of n; LEVELS: of P.  Three CTAs per SM: without the limit the compiler keeps so many
+// rows in flight per thread that one fits, and P = 24, S = 4, D = 5025045 took 407 instead of
+// 190 us.)
+template <class A, int BITS, int LEVELS>
+__global__ void __launch_bounds__(256, LEVELS == 4 ? 4 : LEVELS == 8 ? 3 : 1) k_local_global_any(const float* src, int64_t src_ld, int n,
+                                                          float* w, int64_t ld, int64_t cols, int S,
                                                           int G) {
   grid_dep_wait();
-  const int64_t c = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (c >= cols_v) return;
-  V* p = w + c;
-  const V* q = src + c;
-  V stack[32];
-  int64_t i = 0;   // index of the next pushed value of the global sequence
+  const A a(cols);
+  if (a.live == 0) return;
+  Counter<typename A::V, LEVELS> cnt;
   for (int g = 0; g < G; ++g) {
-    const V m = vdiv(tree_any(q + static_cast<int64_t>(g) * n * src_ld_v, src_ld_v, n),
-                     static_cast<float>(S));
-    for (int r = 0; r < S; ++r, ++i) {
-      V x = m;
-      int l = 0;
-      while ((i >> l) & 1) {
-        x = vadd(stack[l], x);
-        ++l;
-      }
-      stack[l] = x;
+    const typename A::V m =
+        vdiv(tree_rows<BITS, false>(a, src + static_cast<int64_t>(g) * n * src_ld, src_ld, n),
+             static_cast<float>(S));
+    for (int i = g * S, end = i + S; i < end;) {
+      int l = 31 - __clz(end - i);
+      if (i != 0) l = min(l, __ffs(i) - 1);
+      typename A::V x = m;
+      for (int k = 0; k < l; ++k) x = vadd(x, x);
+      cnt.push(i, l, x);
+      i += 1 << l;
     }
   }
   const int total = S * G;
-  V acc{};
-  bool have = false;
-  for (int l = 0; l < 32; ++l) {
-    if ((total >> l) & 1) {
-      acc = have ? vadd(stack[l], acc) : stack[l];
-      have = true;
-    }
-  }
-  store_rows(p, ld_v, total, vdiv(acc, static_cast<float>(total)));
+  const typename A::V m = vdiv(cnt.total(total, typename A::V{}, false), static_cast<float>(total));
+#pragma unroll 8
+  for (int i = 0; i < total; ++i) a.store(w + static_cast<int64_t>(i) * ld, m);
 }
 
 constexpr int kThreads = 256;
@@ -317,15 +441,6 @@ bool mean_pow2_to_dispatch(int log, const float4* w, int64_t ld_v, int64_t cols_
     case 7: launch_mean_pow2_to<7>(w, ld_v, cols_v, groups, div, out, out_ld_v, s); return true;
     default: return false;
   }
-}
-
-template <class V>
-void launch_mean_any_to(const V* w, int64_t ld_v, int64_t cols_v, int n, int64_t groups, float div,
-                        V* out, int64_t out_ld_v, cudaStream_t s) {
-  dim3 grid(static_cast<unsigned>((cols_v + kThreads - 1) / kThreads),
-            static_cast<unsigned>(groups));
-  launch_pdl(k_mean_any_to<V>, grid, dim3(kThreads), 0, s, false, 1, w, ld_v, cols_v, n, div, out,
-             out_ld_v);
 }
 
 bool mean_pow2_dispatch(int log, float4* w, int64_t ld_v, int64_t cols_v, int64_t groups,
@@ -394,42 +509,88 @@ bool lg_dispatch(int logq, int logs, int logg, const float4* src, int64_t src_ld
   }
 }
 
-template <class V>
-void launch_mean_any(V* w, int64_t ld_v, int64_t cols_v, int n, int64_t groups,
-                     cudaStream_t s) {
-  dim3 grid(static_cast<unsigned>((cols_v + kThreads - 1) / kThreads),
-            static_cast<unsigned>(groups));
-  launch_pdl(k_mean_any<V>, grid, dim3(kThreads), 0, s, false, 1, w, ld_v, cols_v, n);
+// Grid of the generic kernels: 256 threads of A::kCols columns each.
+template <class A>
+dim3 any_grid(int64_t cols, int64_t groups) {
+  return dim3(static_cast<unsigned>((cols + 256 * A::kCols - 1) / (256 * A::kCols)),
+              static_cast<unsigned>(groups));
 }
 
-template <class V>
-void launch_lg_any(const V* src, int64_t src_ld_v, int n, V* w, int64_t ld_v, int64_t cols_v, int S,
+template <class A, bool kTo>
+void launch_mean_any(const float* src, int64_t ld, int64_t cols, int n, int64_t groups, float div,
+                     float* dst, int64_t dst_ld, cudaStream_t s) {
+  launch_pdl(n < 16 ? k_mean_any<A, 4, kTo> : k_mean_any<A, 8, kTo>, any_grid<A>(cols, groups),
+             dim3(256), 0, s, false, 1, src, ld, cols, n, div, dst, dst_ld);
+}
+
+// Four columns per thread while that gives every SM two CTAs.
+bool spread_wide(int64_t cols, int64_t groups) { return cols * groups >= 2 * 152 * 1024; }
+
+template <bool kTo>
+void mean_any_dispatch(bool vec, const float* src, int64_t ld, int64_t cols, int n, int64_t groups,
+                       float div, float* dst, int64_t dst_ld, cudaStream_t s) {
+  if (n >= 256)     // (one column per thread: 27 float partials fit in registers)
+    launch_pdl(k_mean_any<Single, 31, kTo>, any_grid<Single>(cols, groups), dim3(256), 0, s, false, 1,
+               src, ld, cols, n, div, dst, dst_ld);
+  else if (vec)
+    launch_mean_any<Quad, kTo>(src, ld, cols, n, groups, div, dst, dst_ld, s);
+  else if (spread_wide(cols, groups))
+    launch_mean_any<Spread, kTo>(src, ld, cols, n, groups, div, dst, dst_ld, s);
+  else
+    launch_mean_any<Single, kTo>(src, ld, cols, n, groups, div, dst, dst_ld, s);
+}
+
+template <class A>
+void launch_lg_any(const float* src, int64_t src_ld, int n, float* w, int64_t ld, int64_t cols, int S,
                    int G, cudaStream_t s) {
-  dim3 grid(static_cast<unsigned>((cols_v + kThreads - 1) / kThreads));
-  launch_pdl(k_local_global_any<V>, grid, dim3(kThreads), 0, s, false, 1, src, src_ld_v, n, w, ld_v,
-             cols_v, S, G);
+  launch_pdl(S * G < 16 ? k_local_global_any<A, 4, 4> : n < 16 ? k_local_global_any<A, 4, 8>
+                                                          : k_local_global_any<A, 8, 8>,
+             any_grid<A>(cols, 1), dim3(256), 0, s, false, 1, src, src_ld, n, w, ld, cols, S, G);
+}
+
+void lg_any_dispatch(bool vec, const float* src, int64_t src_ld, int n, float* w, int64_t ld,
+                     int64_t cols, int S, int G, cudaStream_t s) {
+  if (static_cast<int64_t>(S) * G >= 256)
+    launch_pdl(k_local_global_any<Single, 31, 31>, any_grid<Single>(cols, 1), dim3(256), 0, s, false, 1, src,
+               src_ld, n, w, ld, cols, S, G);
+  else if (vec)
+    launch_lg_any<Quad>(src, src_ld, n, w, ld, cols, S, G, s);
+  else if (spread_wide(cols, 1))
+    launch_lg_any<Spread>(src, src_ld, n, w, ld, cols, S, G, s);
+  else
+    launch_lg_any<Single>(src, src_ld, n, w, ld, cols, S, G, s);
 }
 
 }  // namespace
 
-// Vector path for the 16-byte aligned bulk, scalar generic path for the tail.
+// Whether every row starts on 16 bytes.
 static bool vec_ok(const float* w, int64_t ld) {
   return (reinterpret_cast<uintptr_t>(w) % 16 == 0) && (ld % 4 == 0);
 }
+
+// The power-of-two kernels take aligned rows of whole quads; everything else (other group
+// sizes, other alignments) goes to the generic kernels.  A partial last quad does too, in one
+// launch, unless the matrix is so large that the power-of-two kernels' unrolled trees of 16
+// rows or more are worth a second launch for the last columns: P = 128, S = 32, D = 4000001
+// local 607 against 626 us, local + global 686 against 777; P = 64, S = 8, D = 1000001
+// local 80.7 against 76.9 us, global 114 against 103, local + global 124 against 122.
+constexpr int64_t kTailLaunch = int64_t(256) << 20;   // values in the matrix
+static bool tail_launch(int64_t rows, int64_t D) { return D % 4 != 0 && rows * D >= kTailLaunch; }
 
 cudaError_t launch_group_mean(float* w, int64_t P, int64_t n, int64_t D, int64_t ld,
                               cudaStream_t s) {
   if (D == 0 || n == 1) return cudaSuccess;   // a mean of one row is that row
   const int64_t groups = P / n;
-  int64_t head = 0;
-  if (vec_ok(w, ld) && D >= 4) {
+  const bool vec = vec_ok(w, ld);
+  const int log = ilog2_exact(n);
+  const bool tail = n >= 16 && tail_launch(P, D);
+  int64_t head = 0;                           // columns done by a power-of-two kernel
+  if (vec && (D % 4 == 0 || tail) && log >= 1 &&
+      mean_pow2_dispatch(log, reinterpret_cast<float4*>(w), ld / 4, D / 4, groups, s))
     head = D & ~int64_t(3);
-    float4* w4 = reinterpret_cast<float4*>(w);
-    const int log = ilog2_exact(n);
-    if (!(log >= 1 && mean_pow2_dispatch(log, w4, ld / 4, head / 4, groups, s)))
-      launch_mean_any<float4>(w4, ld / 4, head / 4, static_cast<int>(n), groups, s);
-  }
-  if (head < D) launch_mean_any<float>(w + head, ld, D - head, static_cast<int>(n), groups, s);
+  if (head < D)
+    mean_any_dispatch<false>(vec, w + head, ld, D - head, static_cast<int>(n), groups,
+                             static_cast<float>(n), w + head, ld, s);
   return cudaGetLastError();
 }
 
@@ -442,19 +603,12 @@ cudaError_t launch_group_sum_mean_to(const float* w, int64_t rows, int64_t n, in
                                      float div, float* out, int64_t out_ld, cudaStream_t s) {
   if (D == 0) return cudaSuccess;
   const int64_t groups = rows / n;
-  int64_t head = 0;
-  if (vec_ok(w, ld) && vec_ok(out, out_ld) && D >= 4) {
-    head = D & ~int64_t(3);
-    const float4* w4 = reinterpret_cast<const float4*>(w);
-    float4* o4 = reinterpret_cast<float4*>(out);
-    const int log = ilog2_exact(n);
-    if (!(log >= 0 && mean_pow2_to_dispatch(log, w4, ld / 4, head / 4, groups, div, o4, out_ld / 4, s)))
-      launch_mean_any_to<float4>(w4, ld / 4, head / 4, static_cast<int>(n), groups, div, o4,
-                                 out_ld / 4, s);
-  }
-  if (head < D)
-    launch_mean_any_to<float>(w + head, ld, D - head, static_cast<int>(n), groups, div, out + head,
-                              out_ld, s);
+  const bool vec = vec_ok(w, ld) && vec_ok(out, out_ld);
+  const int log = ilog2_exact(n);
+  if (!(vec && D % 4 == 0 && log >= 0 &&
+        mean_pow2_to_dispatch(log, reinterpret_cast<const float4*>(w), ld / 4, D / 4, groups, div,
+                              reinterpret_cast<float4*>(out), out_ld / 4, s)))
+    mean_any_dispatch<true>(vec, w, ld, D, static_cast<int>(n), groups, div, out, out_ld, s);
   return cudaGetLastError();
 }
 
@@ -472,20 +626,16 @@ cudaError_t launch_local_global_from_groups(const float* src, int64_t src_ld, in
                                             cudaStream_t s) {
   if (D == 0) return cudaSuccess;
   const int64_t G = P / S, n = S / Q;
+  const bool vec = vec_ok(w, ld) && vec_ok(src, src_ld);
+  const int logq = ilog2_exact(Q), logs = ilog2_exact(S), logg = ilog2_exact(G);
   int64_t head = 0;
-  if (vec_ok(w, ld) && vec_ok(src, src_ld) && D >= 4) {
+  if (vec && (D % 4 == 0 || tail_launch(P, D)) && logq >= 0 && logs >= 1 && logg >= 0 &&
+      lg_dispatch(logq, logs, logg, reinterpret_cast<const float4*>(src), src_ld / 4,
+                  reinterpret_cast<float4*>(w), ld / 4, D / 4, s))
     head = D & ~int64_t(3);
-    float4* w4 = reinterpret_cast<float4*>(w);
-    const float4* s4 = reinterpret_cast<const float4*>(src);
-    const int logq = ilog2_exact(Q), logs = ilog2_exact(S), logg = ilog2_exact(G);
-    if (!(logq >= 0 && logs >= 1 && logg >= 0 &&
-          lg_dispatch(logq, logs, logg, s4, src_ld / 4, w4, ld / 4, head / 4, s)))
-      launch_lg_any<float4>(s4, src_ld / 4, static_cast<int>(n), w4, ld / 4, head / 4,
-                            static_cast<int>(S), static_cast<int>(G), s);
-  }
   if (head < D)
-    launch_lg_any<float>(src + head, src_ld, static_cast<int>(n), w + head, ld, D - head,
-                         static_cast<int>(S), static_cast<int>(G), s);
+    lg_any_dispatch(vec, src + head, src_ld, static_cast<int>(n), w + head, ld, D - head,
+                    static_cast<int>(S), static_cast<int>(G), s);
   return cudaGetLastError();
 }
 

@@ -76,6 +76,23 @@ def test_strided_and_misaligned(offset, ld_extra):
         assert np.array_equal(_bits(got), _bits(_oracle(w, op, S)))
 
 
+# The generic kernels at the edges of their dispatch: rows of 1 to 4 columns past a quad, a
+# CTA or the four-columns-per-thread limit (152 x 2048 columns), aligned rows with a partial
+# last quad, unaligned rows; group sizes around 16 (blocks of 16 rows) and 256 (the register
+# variants), none of them powers of two, and clusters whose copies end inside a block of the
+# global tree.
+@pytest.mark.parametrize("P,S,D,offset,ld_extra", [
+    (6, 3, 5, 0, 3), (6, 3, 1025, 0, 3), (12, 6, 1023, 1, 0), (15, 5, 1022, 0, 2), (17, 17, 1021, 0, 7),
+    (30, 15, 770, 0, 6), (34, 17, 258, 3, 0), (48, 16, 515, 0, 1), (96, 3, 259, 0, 1), (100, 20, 301, 2, 1),
+    (250, 25, 130, 0, 2), (255, 51, 67, 0, 0), (256, 64, 37, 1, 0), (300, 100, 33, 0, 3), (514, 257, 9, 0, 0),
+    (4100, 4100, 6, 0, 2), (3, 3, 311297, 0, 0), (4, 2, 311299, 1, 0), (6, 2, 155649, 0, 0)])
+def test_generic_kernels(P, S, D, offset, ld_extra):
+    w = replica_matrix(P, D, seed=P + D).numpy()
+    for op in ("local", "global", "local_global"):
+        got = _gpu(w, op, S, ld=D + ld_extra, offset=offset)
+        assert np.array_equal(_bits(got), _bits(_oracle(w, op, S))), op
+
+
 def test_edge_values():
     P, S, D = 8, 2, 64
     rng = np.random.default_rng(5)
