@@ -28,7 +28,7 @@ constexpr int kGA = kHeadMaxC + 8;            // g_q   [b][c] row stride (bf16)
 constexpr int kGT = 64 + 8;                   // g_q^T [c][b] row stride (bf16)
 
 __device__ __forceinline__ const __nv_bfloat16* head_row(const HeadArgs& a, int j, int b) {
-  if (a.x_rows) return a.H + (static_cast<int64_t>(j) * a.N + (a.row0 + b) % a.N) * a.in;
+  if (a.x_rows) return a.H + (static_cast<int64_t>(j) * a.N + wrap_row(a.row0 + b, a.N)) * a.in;
   return a.H + (static_cast<int64_t>(j) * a.Bn + b) * a.pitch_in;
 }
 
@@ -92,7 +92,8 @@ __device__ __forceinline__ void head_body(const HeadArgs& a, uint8_t* smem, int 
   const int C = CT > 0 ? CT : a.C, B = a.B, Bn = a.Bn, in = a.in;
   const int warp = t >> 5, lane = t & 31;
   const int FP = F + kHeadPad;
-  const int k0 = s * F, kc = min(F, in - k0);          // kc > 0, a multiple of 64
+  const int k0 = s * F, kc = min(F, in - k0);          // kc > 0, a multiple of 8
+  const int kp = (kc + 15) & ~15;                       // staged width, zeros from kc on
   __nv_bfloat16* hs = reinterpret_cast<__nv_bfloat16*>(smem);   // [Bn][FP]  H slice
   __nv_bfloat16* wq = hs + Bn * FP;                             // [16][FP]  W_q slice
   float* zp = reinterpret_cast<float*>(wq + kHeadMaxC * FP);    // [64][16]  partial logits
@@ -108,25 +109,25 @@ __device__ __forceinline__ void head_body(const HeadArgs& a, uint8_t* smem, int 
   const int64_t src_row = static_cast<int64_t>(j / a.src_div) * a.ld; // read
   const float* Wr = a.W_src + src_row;
 
-  // ---- 1. stage the slice (padding rows zero) and the labels, form the partial logits
-  const int vpr = kc / 8;                                       // 16-byte vectors per H row
+  // ---- 1. stage the slice (padding zero) and the labels, form the partial logits
+  const int vpr = kp / 8;                                       // 16-byte vectors per H row
   for (int idx = t; idx < Bn * vpr; idx += kHeadThreads) {
     const int b = idx / vpr, v = idx - b * vpr;
     uint4 x = make_uint4(0, 0, 0, 0);
-    if (b < B) x = *reinterpret_cast<const uint4*>(head_row(a, j, b) + k0 + v * 8);
+    if (b < B && v * 8 < kc) x = *reinterpret_cast<const uint4*>(head_row(a, j, b) + k0 + v * 8);
     *reinterpret_cast<uint4*>(hs + b * FP + v * 8) = x;
   }
-  const int wpr = kc / 4;                                       // float4s per W row
+  const int wpr = kp / 4;                                       // float4s per W row
   for (int idx = t; idx < kHeadMaxC * wpr; idx += kHeadThreads) {
     const int c = idx / wpr, v = idx - c * wpr;
     float4 w = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (c < C) w = *reinterpret_cast<const float4*>(Wr + static_cast<int64_t>(c) * in + k0 + v * 4);
+    if (c < C && v * 4 < kc) w = *reinterpret_cast<const float4*>(Wr + static_cast<int64_t>(c) * in + k0 + v * 4);
     __nv_bfloat162* d = reinterpret_cast<__nv_bfloat162*>(wq + c * FP + v * 4);
     d[0] = __floats2bfloat162_rn(w.x, w.y);
     d[1] = __floats2bfloat162_rn(w.z, w.w);
   }
   if (t < kHeadMaxC) bls[t] = t < C ? a.bias_src[src_row + t] : 0.f;
-  if (t >= 64 && t < 64 + B) ys[t - 64] = a.y[static_cast<int64_t>(j) * a.N + (a.row0 + t - 64) % a.N];
+  if (t >= 64 && t < 64 + B) ys[t - 64] = a.y[static_cast<int64_t>(j) * a.N + wrap_row(a.row0 + t - 64, a.N)];
   sync();
   for (int tile = warp; tile < (Bn / 16) * 2; tile += kHeadThreads / 32) {
     const int mt = tile >> 1, nt = tile & 1;                    // 16 samples x 8 classes

@@ -278,7 +278,14 @@ int plan_layout(hier_avg* h) {
       max_tiles = std::max(max_tiles, std::max(ftiles, btiles) * P);
     }
     h->fused_xent = h->dims[L] <= 128;
-    h->head = ha::head_supported(h->dims[L], h->dims[L - 1], static_cast<int>(B), h->P);
+    // Last layers of up to 16 classes run as one kernel.  Where the width is no multiple of
+    // 64 that replaces the tensor-core forward and backward with their partly filled tiles:
+    // 264-136-200-13 (P = 6, B = 20) 55 -> 43 us per step, one-layer 784-10 (P = 24, B = 64)
+    // 43 -> 15 us.  Wide layers after hidden ones keep the tensor-core kernels, whose tiles
+    // are nearly full there (2512 -> 10 behind 3072-512, P = 4: 1.6 % of the step).
+    const int64_t wl = h->dims[L - 1];
+    h->head = (wl % 64 == 0 || L == 1 || wl <= 1024) &&
+              ha::head_supported(h->dims[L], h->dims[L - 1], static_cast<int>(B), h->P);
     h->off_part = take(part_bytes);
     h->off_cnt = take(max_tiles * 4);
     h->off_dyn = take(16);
@@ -585,7 +592,7 @@ int do_step(hier_avg* h, bool h1_ready = false, bool fuse_next = false, bool* fu
     // around the end of the data set; then the rows are gathered first.
     const int64_t r0 = h->cursor % h->N;   // this step's batch: rows r0 .. (mod N)
     const bool x_direct = r0 + B <= h->N;
-    if (!x_direct) {
+    if (!x_direct && !(h->head && L == 1)) {   // (the head kernel wraps its rows itself)
       rc = h->timed(HA_KERNEL_GATHER, double(P) * B * d0 * 2 * 3, 0.0, [&] {
         return ha::launch_gather_bf16(static_cast<const __nv_bfloat16*>(h->X), h->N, d0, B, h->Bn,
                                       h->pitch[0], r0, P, h->wsp<__nv_bfloat16>(h->off_H[0]), s);

@@ -16,6 +16,13 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
 
+// r mod N for a row index r >= 0 of a batch: almost always below N, or one turn past it (a
+// 64-bit modulo is ~100 instructions).
+__device__ __forceinline__ int64_t wrap_row(int64_t r, int64_t N) {
+  if (r < N) return r;
+  return r - N < N ? r - N : r % N;
+}
+
 // ---------------------------------------------------------------- mbarrier
 __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count));

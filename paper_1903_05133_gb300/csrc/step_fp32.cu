@@ -39,13 +39,6 @@ __device__ __forceinline__ void cp_async_wait() {
   asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
-// r mod N for a row index r >= 0 of a batch: almost always below N, or one turn past it (a
-// 64-bit modulo is ~100 instructions).
-__device__ __forceinline__ int64_t wrap_row(int64_t r, int64_t N) {
-  if (r < N) return r;
-  return r - N < N ? r - N : r % N;
-}
-
 // Columns [k0, k0 + W) of rows [0, R) into dst (row pitch `pitch` floats) by 256 threads;
 // row(r) is the address of row r's column 0 (nullptr: zeros), columns from kmax on are
 // zeros.  vec: every row starts on 16 bytes and kmax is a multiple of 4.

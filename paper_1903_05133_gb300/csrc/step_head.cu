@@ -42,7 +42,7 @@ cudaError_t launch_cluster(const HeadArgs& a, int P, cudaStream_t s) {
 }  // namespace
 
 bool head_supported(int C, int in, int B, int P) {
-  return C <= kHeadMaxC && in % 64 == 0 && B <= 64 &&
+  return C <= kHeadMaxC && B <= 64 &&
          (in + head_slice(in, P) - 1) / head_slice(in, P) <= kHeadClusterMax &&
          head_smem_bytes(in, P, 64) <= 200 * 1024;
 }

@@ -226,8 +226,8 @@ SMALL_FP32 = configs.Workload("tiny_mlp_fp32", P=4, S=2, K1=2, K2=2, rounds=1,
 
 # Last-layer paths: CUDA-core head kernels (<= 16 classes; SMALL_BF16, SOFTMAX_BF16 which
 # reads X directly, the 16-learner MLP, HEAD_C13 with a class count that is not the
-# specialised 10), tensor-core forward with the CE in its
-# epilogue (RAGGED_BF16: 13 classes over a 200-wide ragged input; WIDE_SOFTMAX_BF16),
+# specialised 10, RAGGED_BF16: 13 classes over a 200-wide ragged input), tensor-core forward
+# with the CE in its epilogue (WIDE_SOFTMAX_BF16),
 # and the standalone CE kernel (MANY_CLASSES_BF16: 300 classes over 3 tiles).
 STEP_CASES = [configs.SOFTMAX_P4, SMALL_FP32, SMALL_BF16, SOFTMAX_BF16, HEAD_C13,
               WIDE_SOFTMAX_BF16, RAGGED_BF16, MANY_CLASSES_BF16, configs.MLP512_P16, FUSE_PIECES,
@@ -715,3 +715,25 @@ def test_fp32_steps_in_one_launch(w, G):
     assert ha1.get_step() == ha2.get_step() == 2 * n
     assert torch.equal(ha1.params.view(torch.int32), ha2.params.view(torch.int32))
     assert torch.equal(ha1.losses(), ha2.losses())
+
+
+# The one-kernel last layer on input widths that are no multiple of 64: the narrowest (8
+# features, half an MMA step), a width over 4 and over 8 CTAs whose last slice ends on an
+# odd multiple of 8, one class and 16, a one-layer model whose batches wrap, and a wide
+# one; over 1024 features behind a hidden layer, or 20 classes, stay with the cross-entropy in
+# the forward's epilogue.
+def _head(dims, P, S, B, N):
+    return configs.Workload("head_" + "-".join(map(str, dims)) + f"_P{P}_B{B}", P=P, S=S, K1=2, K2=2, rounds=1,
+                            dims=dims, precision="bf16", N=N, B=B, lr=0.05, sigma_mu=0.1, init="he")
+
+
+HEAD_CASES = [_head((64, 8, 10), 4, 2, 16, 64), _head((136, 200, 13), 6, 3, 20, 50),
+              _head((128, 1000, 16), 24, 4, 33, 132), _head((72, 88, 1), 2, 1, 1, 4),
+              _head((520, 10), 4, 4, 24, 50), _head((4104, 16), 2, 2, 64, 256), _head((64, 1032, 16), 2, 2, 64, 256),
+              _head((264, 200, 20), 6, 3, 20, 50)]
+
+
+@pytest.mark.parametrize("w", HEAD_CASES, ids=lambda w: w.name)
+def test_head_widths(w):
+    test_one_step_from_distinct_learners(w)
+    test_literal_sequence_equals_round(w)
