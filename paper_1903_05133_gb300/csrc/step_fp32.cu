@@ -12,9 +12,11 @@
 // multiple of four floats move as 16-byte cp.async copies, others as 4-byte ones.
 // Rounds against 16 x 16-tile kernels with one output per thread and a serial reduction
 // (seven launches per step of a two-layer net): 3072-10 (P = 4, B = 16, 4 steps) 350 -> 29 us,
-// 100-37-10 (P = 4, B = 7, 4 steps) 127 -> 50 us, 3072-512-10 (P = 16, B = 32, 8 steps)
-// 4965 -> 990 us; error against 64 bits the same or smaller (5e-8 at 3072-10, was 1.2e-7).
+// 100-37-10 (P = 4, B = 7, 4 steps) 127 -> 49 us, 3072-512-10 (P = 16, B = 32, 8 steps)
+// 4965 -> 930 us; error against 64 bits the same or smaller (5e-8 at 3072-10, was 1.2e-7;
+// ReLU flips at 3072-512-10 in 6 of 40 seeds' rounds, were in 8).
 #include <cstdint>
+#include <type_traits>
 #include <cuda_runtime.h>
 
 #include "internal.h"
@@ -38,6 +40,33 @@ template <int N>
 __device__ __forceinline__ void cp_async_wait() {
   asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
+
+// ------------------------------------------------------------------ packed FMA
+// Two fp32 FMAs in one instruction, each rounded as fmaf rounds it.  A scalar FFMA of an outer
+// product is held up by the register file (three reads per product): 8 x 8 products per thread
+// in registers ran at 55 TFLOP/s with FFMA, at 65 with pairs.
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ uint64_t pack2(float lo, float hi) {
+  uint64_t d;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(lo), "f"(hi));
+  return d;
+}
+__device__ __forceinline__ float2 unpack2(uint64_t v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+
+// A warp's lanes as 4 (y) x 8 (x) threads of a tile.  A 128-bit shared-memory read takes two
+// cycles when each half-warp's lanes, taken in neighbouring pairs, touch at most 128 bytes,
+// and four otherwise: with y in the lane's lowest bit and highest bit both operands of an
+// outer product do (measured: x = lane & 7 takes four cycles, x = lane >> 1 & 7 two).
+__device__ __forceinline__ int lane_y(int lane) { return (lane >> 4 << 1) | (lane & 1); }
+__device__ __forceinline__ int lane_x(int lane) { return lane >> 1 & 7; }
 
 // Columns [k0, k0 + W) of rows [0, R) into dst (row pitch `pitch` floats) by 256 threads;
 // row(r) is the address of row r's column 0 (nullptr: zeros), columns from kmax on are
@@ -83,11 +112,14 @@ struct WRows {
 // samples x 64 columns.  The eight warps of a CTA split the reduction, not the tile: each
 // warp holds the whole tile (BM = 64: half of its samples) in registers, 8 columns by up
 // to 8 samples per thread, and takes an eighth of every 64-wide chunk of K, so that a
-// chunk's 16-byte shared-memory reads feed 16 FFMAs each (25 % of the shared-memory
+// chunk's 16-byte shared-memory reads feed 16 FFMAs each (half of the shared-memory
 // bandwidth at the FFMA rate).  With few tiles a cluster of up to 8 CTAs shares a tile's
 // chunks.  The partials meet in shared memory and then through distributed shared memory,
 // added in a fixed order (warp, then CTA rank).  Operands arrive by cp.async, three chunks
-// deep.  The forward of 3072 -> 512 (P = 16, B = 32) takes 58 us, 28 TFLOP/s.
+// deep.  The forward of 3072 -> 512 (P = 16, B = 32) takes 56 us, 29 TFLOP/s: 45 us of products
+// and reductions on the SMs with two CTAs (48 chunks, the average is 40), 26 us of loads, not
+// wholly overlapped.  (A fourth stage took 63 us: what shared memory takes, L1 lacks for the
+// copies in flight.)
 constexpr int kThreads = 256;
 constexpr int kBN = 64;                 // columns of a tile
 constexpr int kKC = 64;                 // reduction chunk
@@ -119,8 +151,8 @@ struct TileArgs {
 // kDx false: y[b][o] = sum_k act[b][k] W[o][k]; true: y[b][i] = sum_o act[b][o] W[o][i].
 template <int BM, bool kDx>
 __global__ void __launch_bounds__(kThreads, 2) k_tile_f32(const TileArgs a, int split) {
-  constexpr int WM = BM > 32 ? 2 : 1;   // warps along the samples
-  constexpr int MW = BM / WM;           // samples of a warp
+  constexpr int MW = BM < 32 ? BM : 32;   // samples of a warp
+  constexpr int WM = BM / MW;           // warps along the samples
   constexpr int TM = MW / 4;            // samples of a thread
   constexpr int KS = 8 / WM;            // warps along the reduction
   constexpr int KW = kKC / KS;          // reduction indices of a warp in a chunk
@@ -151,12 +183,17 @@ __global__ void __launch_bounds__(kThreads, 2) k_tile_f32(const TileArgs a, int 
       load_rows<kKC, kBN>(ws, kKP, c * kKC, a.in, a.vec_w, a.W, t,
                           WRows{W + static_cast<int64_t>(n0) * a.in, a.in, a.out - n0});
   };
-  const int ks = warp % KS, wm = warp / KS, ly = lane >> 3, lx = lane & 7;
-  float acc[TM][8];
+  const int ks = warp % KS, wm = warp / KS, ly = lane_y(lane), lx = lane_x(lane);
+  // dX: pairs of columns, which lie side by side in its weight chunk.  The forward's pairs
+  // would be even and odd indices of the reduction, with half the samples per thread and 1.5
+  // times the shared-memory reads per product: no faster (56.5 against 56 us), so scalars.
+  constexpr int NA = kDx ? 4 : 8;
+  using Acc = std::conditional_t<kDx, uint64_t, float>;
+  Acc acc[TM][NA];
 #pragma unroll
   for (int i = 0; i < TM; ++i)
 #pragma unroll
-    for (int n = 0; n < 8; ++n) acc[i][n] = 0.f;
+    for (int n = 0; n < NA; ++n) acc[i][n] = 0;
 
 #pragma unroll
   for (int s = 0; s < kStages - 1; ++s) {
@@ -172,42 +209,41 @@ __global__ void __launch_bounds__(kThreads, 2) k_tile_f32(const TileArgs a, int 
     const float* ws = sm + (it % kStages) * tile_stage_floats(BM) + BM * kKP;
 #pragma unroll
     for (int k = 0; k < KW; k += 4) {
-      float4 av[TM];
-#pragma unroll
-      for (int i = 0; i < TM; ++i) av[i] = *reinterpret_cast<const float4*>(as + 4 * i * kKP + k);
       if constexpr (kDx) {
+        float4 av[TM];
+#pragma unroll
+        for (int i = 0; i < TM; ++i) av[i] = *reinterpret_cast<const float4*>(as + 4 * i * kKP + k);
 #pragma unroll
         for (int kk = 0; kk < 4; ++kk) {
           const float* wr = ws + (ks * KW + k + kk) * kBN + 4 * lx;
-          const float4 w0 = *reinterpret_cast<const float4*>(wr);
-          const float4 w1 = *reinterpret_cast<const float4*>(wr + 32);
+          const ulonglong2 w0 = *reinterpret_cast<const ulonglong2*>(wr);
+          const ulonglong2 w1 = *reinterpret_cast<const ulonglong2*>(wr + 32);
 #pragma unroll
           for (int i = 0; i < TM; ++i) {
             const float x = kk == 0 ? av[i].x : kk == 1 ? av[i].y : kk == 2 ? av[i].z : av[i].w;
-            acc[i][0] = fmaf(x, w0.x, acc[i][0]);
-            acc[i][1] = fmaf(x, w0.y, acc[i][1]);
-            acc[i][2] = fmaf(x, w0.z, acc[i][2]);
-            acc[i][3] = fmaf(x, w0.w, acc[i][3]);
-            acc[i][4] = fmaf(x, w1.x, acc[i][4]);
-            acc[i][5] = fmaf(x, w1.y, acc[i][5]);
-            acc[i][6] = fmaf(x, w1.z, acc[i][6]);
-            acc[i][7] = fmaf(x, w1.w, acc[i][7]);
+            const uint64_t xx = pack2(x, x);
+            acc[i][0] = fma2(xx, w0.x, acc[i][0]);
+            acc[i][1] = fma2(xx, w0.y, acc[i][1]);
+            acc[i][2] = fma2(xx, w1.x, acc[i][2]);
+            acc[i][3] = fma2(xx, w1.y, acc[i][3]);
           }
         }
       } else {
-        float4 wv[8];
+        float4 av[TM];
 #pragma unroll
-        for (int n = 0; n < 8; ++n)
-          wv[n] = *reinterpret_cast<const float4*>(ws + (lx + 8 * n) * kKP + ks * KW + k);
+        for (int i = 0; i < TM; ++i) av[i] = *reinterpret_cast<const float4*>(as + 4 * i * kKP + k);
 #pragma unroll
-        for (int i = 0; i < TM; ++i)
+        for (int n = 0; n < 8; ++n) {
+          const float4 wv = *reinterpret_cast<const float4*>(ws + (lx + 8 * n) * kKP + ks * KW + k);
 #pragma unroll
-          for (int n = 0; n < 8; ++n) {
-            acc[i][n] = fmaf(av[i].x, wv[n].x, acc[i][n]);
-            acc[i][n] = fmaf(av[i].y, wv[n].y, acc[i][n]);
-            acc[i][n] = fmaf(av[i].z, wv[n].z, acc[i][n]);
-            acc[i][n] = fmaf(av[i].w, wv[n].w, acc[i][n]);
-          }
+          for (int i = 0; i < TM; ++i) acc[i][n] = fmaf(av[i].x, wv.x, acc[i][n]);
+#pragma unroll
+          for (int i = 0; i < TM; ++i) acc[i][n] = fmaf(av[i].y, wv.y, acc[i][n]);
+#pragma unroll
+          for (int i = 0; i < TM; ++i) acc[i][n] = fmaf(av[i].z, wv.z, acc[i][n]);
+#pragma unroll
+          for (int i = 0; i < TM; ++i) acc[i][n] = fmaf(av[i].w, wv.w, acc[i][n]);
+        }
       }
     }
   }
@@ -219,13 +255,13 @@ __global__ void __launch_bounds__(kThreads, 2) k_tile_f32(const TileArgs a, int 
 #pragma unroll
     for (int i = 0; i < TM; ++i) {
       if constexpr (kDx) {
-        *reinterpret_cast<float4*>(red + 4 * i * kRP + 4 * lx) =
-            make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
-        *reinterpret_cast<float4*>(red + 4 * i * kRP + 32 + 4 * lx) =
-            make_float4(acc[i][4], acc[i][5], acc[i][6], acc[i][7]);
+        *reinterpret_cast<ulonglong2*>(red + 4 * i * kRP + 4 * lx) = make_ulonglong2(acc[i][0], acc[i][1]);
+        *reinterpret_cast<ulonglong2*>(red + 4 * i * kRP + 32 + 4 * lx) = make_ulonglong2(acc[i][2], acc[i][3]);
       } else {
 #pragma unroll
-        for (int n = 0; n < 8; ++n) red[4 * i * kRP + lx + 8 * n] = acc[i][n];
+        for (int n = 0; n < 8; ++n) {
+          red[4 * i * kRP + lx + 8 * n] = acc[i][n];
+        }
       }
     }
   }
@@ -286,8 +322,8 @@ __global__ void __launch_bounds__(kThreads, 2) k_tile_f32(const TileArgs a, int 
 // chain per weight) and, in the first input tile, b_l -= lr * sum_b dZ.  CTA = 64 outputs x
 // 128 inputs, thread = 8 x 8 of them; the weights are loaded into registers before the
 // batch arrives, so their latency hides behind the products.  Samples go in chunks of 32
-// through two cp.async stages.  3072 -> 512 (P = 16, B = 32): 57 us, 3.5 TB/s, 28 TFLOP/s
-// (61 us with a 64-bit modulo per batch row).
+// through two cp.async stages.  3072 -> 512 (P = 16, B = 32): 48 us, 4.2 TB/s, 33 TFLOP/s
+// (57 us with scalar FFMAs and lanes 4 x 8 in order, 55 with samples unrolled by two).
 constexpr int kDwThreads = 128;
 constexpr int kDwO = 64, kDwI = 128, kDwB = 32;
 constexpr int kDwStage = kDwB * (kDwO + kDwI);
@@ -308,7 +344,7 @@ struct DwArgs {
 template <bool kVec>           // a.vec_h: thread columns 4 lx .. 4 lx + 3 (+ 32), else lx + 8 n
 __global__ void __launch_bounds__(kDwThreads, 3) k_dw_f32(const DwArgs a) {
   extern __shared__ __align__(16) float sm[];
-  const int t = threadIdx.x, warp = t >> 5, lane = t & 31, ly = lane >> 3, lx = lane & 7;
+  const int t = threadIdx.x, warp = t >> 5, lane = t & 31, ly = lane_y(lane), lx = lane_x(lane);
   const int i0 = blockIdx.x * kDwI, o0 = blockIdx.y * kDwO;
   const int64_t j = blockIdx.z;
   grid_dep_wait();
@@ -368,11 +404,11 @@ __global__ void __launch_bounds__(kDwThreads, 3) k_dw_f32(const DwArgs a) {
         w[e][n] = orow && i0 + col(n) < a.in ? Wj[static_cast<int64_t>(e) * a.in + col(n)] : 0.f;
     }
   }
-  float acc[8][8];
+  uint64_t acc[8][4];                  // columns (0, 1), (2, 3), ... of each output
 #pragma unroll
   for (int e = 0; e < 8; ++e)
 #pragma unroll
-    for (int n = 0; n < 8; ++n) acc[e][n] = 0.f;
+    for (int n = 0; n < 4; ++n) acc[e][n] = 0;
   float db = 0.f;
   for (int c = 0; c < nb; ++c) {
     if (c + 1 < nb) load(c + 1, (c + 1) & 1);
@@ -383,20 +419,23 @@ __global__ void __launch_bounds__(kDwThreads, 3) k_dw_f32(const DwArgs a) {
     const float* hs = zs + kDwB * kDwO;
     const int rows = a.B - c * kDwB < kDwB ? a.B - c * kDwB : kDwB;
     for (int r = 0; r < rows; ++r) {
-      float z[8], h[8];
+      float z[8];
+      uint64_t h[4];
       *reinterpret_cast<float4*>(z) = *reinterpret_cast<const float4*>(zs + r * kDwO + ow);
       *reinterpret_cast<float4*>(z + 4) = *reinterpret_cast<const float4*>(zs + r * kDwO + ow + 4);
       if constexpr (kVec) {
-        *reinterpret_cast<float4*>(h) = *reinterpret_cast<const float4*>(hs + r * kDwI + col(0));
-        *reinterpret_cast<float4*>(h + 4) = *reinterpret_cast<const float4*>(hs + r * kDwI + col(4));
+        *reinterpret_cast<ulonglong2*>(h) = *reinterpret_cast<const ulonglong2*>(hs + r * kDwI + col(0));
+        *reinterpret_cast<ulonglong2*>(h + 2) = *reinterpret_cast<const ulonglong2*>(hs + r * kDwI + col(4));
       } else {
 #pragma unroll
-        for (int n = 0; n < 8; ++n) h[n] = hs[r * kDwI + col(n)];
+        for (int n = 0; n < 4; ++n) h[n] = pack2(hs[r * kDwI + col(2 * n)], hs[r * kDwI + col(2 * n + 1)]);
       }
 #pragma unroll
-      for (int e = 0; e < 8; ++e)
+      for (int e = 0; e < 8; ++e) {
+        const uint64_t zz = pack2(z[e], z[e]);
 #pragma unroll
-        for (int n = 0; n < 8; ++n) acc[e][n] = fmaf(z[e], h[n], acc[e][n]);
+        for (int n = 0; n < 4; ++n) acc[e][n] = fma2(zz, h[n], acc[e][n]);
+      }
     }
     if (blockIdx.x == 0 && t < kDwO)
       for (int r = 0; r < rows; ++r) db = __fadd_rn(db, zs[r * kDwO + t]);
@@ -406,7 +445,11 @@ __global__ void __launch_bounds__(kDwThreads, 3) k_dw_f32(const DwArgs a) {
   for (int e = 0; e < 8; ++e) {
     if (o0 + ow + e >= a.out) break;
 #pragma unroll
-    for (int n = 0; n < 8; ++n) w[e][n] = __fsub_rn(w[e][n], __fmul_rn(a.lr, acc[e][n]));
+    for (int n = 0; n < 8; n += 2) {
+      const float2 g = unpack2(acc[e][n / 2]);
+      w[e][n] = __fsub_rn(w[e][n], __fmul_rn(a.lr, g.x));
+      w[e][n + 1] = __fsub_rn(w[e][n + 1], __fmul_rn(a.lr, g.y));
+    }
     if constexpr (kVec) {
 #pragma unroll
       for (int n = 0; n < 8; n += 4)
