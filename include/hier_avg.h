@@ -238,7 +238,7 @@ int hier_avg_wait_selftest(hier_avg* h, int64_t limit_us);
 #define HA_KERNEL_BACKWARD      3   /* fused dX + dW + SGD update            */
 #define HA_KERNEL_LOCAL_AVG     4
 #define HA_KERNEL_GLOBAL_AVG    5   /* fused last local + global average     */
-#define HA_KERNEL_HEAD          6   /* fused last layer (<= 16 classes)      */
+#define HA_KERNEL_HEAD          6   /* fused last layer (<= 16 classes), or whole steps of a small net */
 #define HA_KERNEL_UPDATE_FORWARD 7  /* first-layer update + next forward     */
 #define HA_KERNEL_KINDS         8
 int hier_avg_profile(hier_avg* h, int enable);

@@ -90,6 +90,7 @@ struct hier_avg {
   std::vector<int> bwd_whole, bwd_np;         // per layer: whole tiles, tail pieces
   bool fused_xent = false;                    // d_L <= 128: CE in the last forward epilogue
   bool w_stream = true;                       // parameters exceed L2: stream W evict-first
+  bool small = false;                         // whole steps in one launch (either precision)
   bool head = false;                          // d_L <= 16: fused last-layer kernel (either precision)
   // binding
   bool bound = false;
@@ -295,6 +296,8 @@ int plan_layout(hier_avg* h) {
     for (int l = 0; l < L; ++l) h->off_H[l] = take(P * B * h->dims[l] * 4);
     for (int l = 1; l <= L; ++l) h->off_dZ[l] = take(P * B * h->dims[l] * 4);
   }
+  h->small = !(h->head && L == 1) &&
+             ha::small_supported(h->dims.data(), L, static_cast<int>(B), h->P, h->prec == HA_PREC_BF16);
   h->off_Z = take(P * B * h->dims[L] * 4);
   h->off_loss = take(P * 4);
   h->off_err = take(16);
@@ -562,6 +565,37 @@ int do_step_f32(hier_avg* h, int steps) {
   return HA_OK;
 }
 
+// `steps` consecutive steps of a small net (h->small) in one launch.
+int do_steps_small(hier_avg* h, int steps) {
+  const int L = h->L;
+  ha::SmallArgs a{};
+  a.L = L;
+  a.B = h->Bstep;
+  a.steps = steps;
+  double w = 0.0, flops = 0.0;
+  for (int l = 0; l < L; ++l) {
+    a.dims[l] = h->dims[l];
+    a.woff[l] = h->woff[l];
+    a.boff[l] = h->boff[l];
+    w += double(h->dims[l]) * h->dims[l + 1] + h->dims[l + 1];
+    flops += flops_gemm(h, l) * (l > 0 ? 3 : 2) * steps;
+  }
+  a.dims[L] = h->dims[L];
+  a.ld = h->ld;
+  a.N = h->N;
+  a.row0 = h->cursor % h->N;
+  a.lr = h->lr;
+  a.params = h->params;
+  a.X = h->X;
+  a.y = h->y;
+  a.loss = h->loss();
+  // the weights read and written once per launch, the batches once
+  const bool bf16 = h->prec == HA_PREC_BF16;
+  const double bytes = double(h->P) * (8.0 * w + double(steps) * a.B * h->dims[0] * (bf16 ? 2 : 4));
+  return h->timed(HA_KERNEL_HEAD, bytes, flops, [&] { return ha::launch_small(a, bf16, h->P, h->stream); },
+                  "small-net steps");
+}
+
 // One step.  h1_ready: H_1 of this step was written by the previous step's
 // update+forward kernel (skip the first layer's forward).  fuse_next: the caller runs
 // the next step right after this one with nothing in between, so this step may
@@ -581,6 +615,12 @@ int do_step(hier_avg* h, bool h1_ready = false, bool fuse_next = false, bool* fu
   const int L = h->L, P = h->P, B = h->Bstep;
   if (fused) *fused = false;
   h->grp.assign(L, 0);
+  if (h->small) {
+    if (int rc = do_steps_small(h, 1)) return rc;
+    ++h->t;
+    h->cursor += B;
+    return HA_OK;
+  }
   const int q = group_out && h->m_ok ? h->upd_group : 1;
   cudaStream_t s = h->stream;
   int rc;
@@ -994,14 +1034,18 @@ int do_round(hier_avg* h, RowFeed* feed = nullptr) {
   const int G = round_steps(h);
   const bool compact = h->m_ok;
   bool h1_ready = false;
-  // fp32 softmax regression (one layer of at most 16 classes): the steps up to the next
-  // average run in one launch.
-  const bool multi = h->prec != HA_PREC_BF16 && h->head && h->L == 1;
+  // Small nets, and fp32 softmax regression (one layer of at most 16 classes): the steps up
+  // to the next average run in one launch, and the averages write every row.
+  const bool multi = h->small || (h->prec != HA_PREC_BF16 && h->head && h->L == 1);
   for (int r = 1; r <= G; ++r) {
     const int k = r - 1;
     if (multi) {
       const int n = std::min(h->K1 - k % h->K1, G - k);
-      if ((rc = do_step_f32(h, n))) return rc;
+      if (feed && (rc = feed->ensure(k + n - 1))) return rc;
+      if (feed && (rc = h->cuda(cudaStreamWaitEvent(h->stream, feed->ev[k + n - 1], 0),
+                                "round_host: wait for the rows")))
+        return rc;
+      if ((rc = h->small ? do_steps_small(h, n) : do_step_f32(h, n))) return rc;
       h->t += n;
       h->cursor += static_cast<int64_t>(n) * h->Bstep;
       r += n - 1;
@@ -1198,7 +1242,10 @@ int hier_avg_bind(hier_avg* h, float* params_dev, void* workspace_dev, int64_t w
   if (h->prec == HA_PREC_BF16) {
     if ((rc = h->cuda(ha::tc_configure(), "bind: kernel attributes"))) return rc;
     if ((rc = h->cuda(ha::head_configure(), "bind: kernel attributes"))) return rc;
+    if ((rc = h->cuda(ha::small_configure(), "bind: kernel attributes"))) return rc;
     if ((rc = build_maps(h))) return rc;
+  } else if ((rc = h->cuda(ha::small_configure(), "bind: kernel attributes"))) {
+    return rc;
   } else if ((rc = h->cuda(ha::fp32_configure(), "bind: kernel attributes"))) {
     return rc;
   }
@@ -1528,7 +1575,10 @@ extern "C" int hier_avg_step_static(hier_avg* h, float* params_dev, const void* 
   if (h->prec == HA_PREC_BF16) {
     if ((rc = h->cuda(ha::tc_configure(), "step_static: kernel attributes"))) return rc;
     if ((rc = h->cuda(ha::head_configure(), "step_static: kernel attributes"))) return rc;
+    if ((rc = h->cuda(ha::small_configure(), "step_static: kernel attributes"))) return rc;
     if ((rc = build_maps(h))) return rc;
+  } else if ((rc = h->cuda(ha::small_configure(), "step_static: kernel attributes"))) {
+    return rc;
   } else if ((rc = h->cuda(ha::fp32_configure(), "step_static: kernel attributes"))) {
     return rc;
   }

@@ -213,6 +213,33 @@ bool head_supported(int C, int in, int B, int P);
 cudaError_t head_configure();   // raises the dynamic shared-memory limit once
 cudaError_t launch_head(const HeadArgs& a, int P, cudaStream_t s);
 
+// ----------------------------------------------------------------- whole steps of a small net
+constexpr int kSmallLayers = 4;   // layers at most
+constexpr int kSmallC = 32;       // classes at most
+// Float offsets of a CTA's shared memory, per layer l: the slice's columns of W_l (fp32, and
+// rounded to bf16 on the bf16 path), its rows of H_l, and b_l of its neurons.
+struct SmallLayout {
+  int w[kSmallLayers], wq[kSmallLayers], h[kSmallLayers], bias[kSmallLayers];
+  int z[2], dz, own[2], loss, labels, raw, total;
+  int wide;                       // outputs of the widest layer, whole slices
+};
+struct SmallArgs {
+  int L, B, steps;                // `steps` consecutive local steps
+  int dims[kSmallLayers + 1];
+  int64_t woff[kSmallLayers], boff[kSmallLayers];
+  int64_t ld, N, row0;            // row0: first row of the first batch in each learner's data
+  float lr;
+  float* params;                  // learner 0's row
+  const void* X;                  // [P][N][dims[0]] fp32 or bf16
+  const int32_t* y;
+  float* loss;                    // [P], of the last step
+  SmallLayout lay;                // set by the launcher, as is vec: rows in whole, aligned quads
+  int vec;
+};
+bool small_supported(const int* dims, int L, int B, int P, bool bf16);
+cudaError_t small_configure();    // raises the dynamic shared-memory limit once
+cudaError_t launch_small(const SmallArgs& a, bool bf16, int P, cudaStream_t s);
+
 // ----------------------------------------------------------------- fp32 CUDA-core step
 // Buffers: H_l [P][B][d_l] fp32, Z_L [P][B][d_L], dZ_l [P][B][d_l] fp32.
 // A layer's input rows: learner j's batch row b is row (row0 + b) mod N of base + j * stride

@@ -720,20 +720,57 @@ def test_fp32_steps_in_one_launch(w, G):
 # The one-kernel last layer on input widths that are no multiple of 64: the narrowest (8
 # features, half an MMA step), a width over 4 and over 8 CTAs whose last slice ends on an
 # odd multiple of 8, one class and 16, a one-layer model whose batches wrap, and a wide
-# one; over 1024 features behind a hidden layer, or 20 classes, stay with the cross-entropy in
+# one; over 1024 features behind a hidden layer, or 40 classes, stay with the cross-entropy in
 # the forward's epilogue.
 def _head(dims, P, S, B, N):
     return configs.Workload("head_" + "-".join(map(str, dims)) + f"_P{P}_B{B}", P=P, S=S, K1=2, K2=2, rounds=1,
                             dims=dims, precision="bf16", N=N, B=B, lr=0.05, sigma_mu=0.1, init="he")
 
 
-HEAD_CASES = [_head((64, 8, 10), 4, 2, 16, 64), _head((136, 200, 13), 6, 3, 20, 50),
-              _head((128, 1000, 16), 24, 4, 33, 132), _head((72, 88, 1), 2, 1, 1, 4),
-              _head((520, 10), 4, 4, 24, 50), _head((4104, 16), 2, 2, 64, 256), _head((64, 1032, 16), 2, 2, 64, 256),
-              _head((264, 200, 20), 6, 3, 20, 50)]
+HEAD_CASES = [_head((4096, 8, 10), 4, 2, 64, 256), _head((600, 200, 13), 6, 3, 20, 50),
+              _head((128, 1000, 16), 24, 4, 33, 132), _head((4096, 520, 1), 2, 1, 1, 4),
+              _head((3336, 10), 4, 4, 64, 90), _head((4104, 16), 2, 2, 64, 256), _head((64, 1032, 16), 2, 2, 64, 256),
+              _head((264, 200, 40), 6, 3, 20, 50)]
 
 
 @pytest.mark.parametrize("w", HEAD_CASES, ids=lambda w: w.name)
 def test_head_widths(w):
+    test_one_step_from_distinct_learners(w)
+    test_literal_sequence_equals_round(w)
+
+
+# Whole steps of a small net in one launch, several between two averages: one to four layers,
+# widths below the eight slices of a learner and of odd length, 1 to 32 classes, batches of 1
+# to 64 that wrap around the data set (more than once in one launch), a last block shorter
+# than K1, odd clusters.
+def _small(dims, precision, P, S, B, K1, N):
+    return configs.Workload(f"small_{precision}_" + "-".join(map(str, dims)) + f"_P{P}_B{B}", P=P, S=S, K1=K1,
+                            K2=2, rounds=1, dims=dims, precision=precision, N=N, B=B, lr=0.05, sigma_mu=0.1,
+                            init="he")
+
+
+SMALL_CASES = [_small((100, 37, 10), "fp32", 4, 2, 7, 2, 40), _small((5, 3, 2), "fp32", 3, 3, 1, 3, 2),
+               _small((33, 64, 65, 7, 32), "fp32", 6, 2, 33, 2, 50), _small((300, 31), "fp32", 1, 1, 64, 3, 100),
+               _small((264, 136, 200, 13), "bf16", 6, 3, 20, 4, 50), _small((8, 8, 1), "bf16", 2, 2, 1, 2, 1),
+               _small((784, 40, 10), "bf16", 15, 5, 64, 3, 192), _small((136, 104, 88, 72, 32), "bf16", 5, 5, 17, 2, 20),
+               _small((1024, 17), "bf16", 18, 6, 48, 5, 96), _small((1000, 120, 8), "bf16", 16, 4, 16, 2, 64)]
+
+
+@pytest.mark.parametrize("w", SMALL_CASES, ids=lambda w: w.name)
+def test_small_net_steps(w):
+    test_one_step_from_distinct_learners(w)
+    test_free_global_interval_literal_sequence(w, 2 * w.K1 + 1)
+    test_literal_sequence_equals_round(w)
+    test_round_host_matches_device_round(w, 0)
+
+
+# The group-sum and head cases above on nets past the one-launch steps' size, so that quads,
+# pairs with three group sums per cluster, one cluster of all learners and 4 CTAs of the head
+# per learner stay covered.
+@pytest.mark.parametrize("w", [GROUP_S8.replace(dims=(512, 384, 10)), GROUP_S6.replace(dims=(392, 264, 13)),
+                               GROUP_S12_K1.replace(dims=(512, 512, 10)), GROUP_SP.replace(dims=(512, 384, 10)),
+                               HEAD_F128.replace(dims=(512, 320, 10)),
+                               RAGGED_BF16.replace(dims=(520, 264, 328, 13))], ids=lambda w: w.name)
+def test_group_sums_past_small_nets(w):
     test_one_step_from_distinct_learners(w)
     test_literal_sequence_equals_round(w)
