@@ -2767,12 +2767,22 @@ cudaError_t launch_tc_update(const CUtensorMap& w_load, const CUtensorMap& w_sto
                              const CUtensorMap& h_in, const CUtensorMap& dz, const TcBwdArgs& a,
                              int group, cudaStream_t s) {
   // Items of kRun chunks per learner, unless a group of learners then leaves fewer than
-  // 4 items per CTA: then kRun / group chunks per learner (the same work per item).
+  // 4 items per CTA: then kRun / group chunks per learner (the same work per item).  Where even
+  // that leaves fewer than two items per CTA, the run with the least work on the fullest CTA,
+  // half a chunk per item for its H tiles (the items are independent: the same bits).
+  // 784-512-10, P = 2, B = 14, 14 items of 8 chunks: round of 6 steps 126 -> 111 us;
+  // 784-512-512-10, P = 4, B = 32, loop of 2 steps 169 -> 160 us.
   TcBwdArgs b = a;
   const int nc = (a.out + 63) / 64;
+  auto items = [&](int run) { return static_cast<int64_t>(a.n_tiles / group) * ((nc + run - 1) / run); };
+  auto cost = [&](int run) {
+    return (items(run) + a.ctas - 1) / a.ctas * (2 * (run < nc ? run : nc) * group + 1);
+  };
   b.run = kRun;
-  if (group > 1 && static_cast<int64_t>(a.n_tiles / group) * ((nc + kRun - 1) / kRun) < 4 * a.ctas)
-    b.run = kRun / group > 0 ? kRun / group : 1;
+  if (group > 1 && items(kRun) < 4 * a.ctas) b.run = kRun / group > 0 ? kRun / group : 1;
+  if (items(b.run) < 2 * a.ctas)
+    for (int run = b.run / 2; run >= 1; run /= 2)
+      if (cost(run) < cost(b.run)) b.run = run;
   // no CTA waits on another: an ordinary (programmatically serialised) launch
   if (group == 4 && a.Bn <= 32)
     return launch_pdl(k_tc_update<4>, dim3(a.ctas), dim3(upd_threads(4)), updg_smem(4, a.Bn), s, false, 1,
