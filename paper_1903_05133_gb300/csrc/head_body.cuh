@@ -36,6 +36,12 @@ __device__ __forceinline__ void cluster_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;"
                ::: "memory");
 }
+__device__ __forceinline__ void cluster_arrive() {
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() {
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
 // The float at the same shared-memory offset in CTA `rank` of this cluster.
 __device__ __forceinline__ float ld_cluster(const float* p, int rank) {
   const uint32_t la = static_cast<uint32_t>(__cvta_generic_to_shared(p));
@@ -80,7 +86,7 @@ __device__ __forceinline__ int a_col(int l) { return (l >> 4) * 8; }
 
 // Shared memory needed by head_body for slices of F features.
 __host__ __device__ inline int head_body_smem(int F, int Bn) {
-  return (Bn + kHeadMaxC) * (F + kHeadPad) * 2 + 3 * 64 * kHeadMaxC * 4 + 64 * 4 + 64 * 4 +
+  return (Bn + kHeadMaxC) * (F + kHeadPad) * 2 + 2 * 64 * kHeadMaxC * 4 + 64 * 4 + 64 * 4 +
          kHeadMaxC * 4 + 64 * kGA * 2 + kHeadMaxC * kGT * 2;
 }
 
@@ -97,8 +103,7 @@ __device__ __forceinline__ void head_body(const HeadArgs& a, uint8_t* smem, int 
   __nv_bfloat16* hs = reinterpret_cast<__nv_bfloat16*>(smem);   // [Bn][FP]  H slice
   __nv_bfloat16* wq = hs + Bn * FP;                             // [16][FP]  W_q slice
   float* zp = reinterpret_cast<float*>(wq + kHeadMaxC * FP);    // [64][16]  partial logits
-  float* zz = zp + 64 * kHeadMaxC;                              // [64][16]  logits
-  float* gs = zz + 64 * kHeadMaxC;                              // [64][16]  CE gradient (fp32)
+  float* gs = zp + 64 * kHeadMaxC;                              // [64][16]  CE gradient (fp32)
   float* rl = gs + 64 * kHeadMaxC;                              // [64]      per-sample loss
   float* bls = rl + 64;                                         // [16]      b_L before update
   int* ys = reinterpret_cast<int*>(bls + kHeadMaxC);            // [64]      labels
@@ -145,10 +150,33 @@ __device__ __forceinline__ void head_body(const HeadArgs& a, uint8_t* smem, int 
     zp[(r + 8) * kHeadMaxC + cc + 1] = d[3];
   }
 
-  // ---- 2. full logits (partials added in slice order), softmax cross-entropy
+  // ---- 3's first operands: the fp32 values this lane updates, loaded ahead of the barrier.
+  auto load_upd = [&](int nt, float2 (&w32)[2], float2& bp32) {
+    const int f = nt * 8 + (lane & 3) * 2;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int c = (lane >> 2) + 8 * h;
+      w32[h] = c < C ? *reinterpret_cast<const float2*>(Wr + static_cast<int64_t>(c) * in + k0 + f)
+                     : make_float2(0.f, 0.f);
+    }
+    bp32 = (a.has_dx && lane < 4)
+               ? *reinterpret_cast<const float2*>(a.bias_prev_src + src_row + k0 + f)
+               : make_float2(0.f, 0.f);
+  };
+  float2 nw32[2], nbp32;
+  if (warp < kc / 8) load_upd(warp, nw32, nbp32);
+
+  // ---- 2. full logits (partials added in slice order) and softmax cross-entropy: 16 lanes
+  // per sample (one per class slot), every sample's remote loads in flight together, max and
+  // sum of exponentials by butterflies over the sample's lanes.
   cluster_sync();
-  for (int pr = t; pr < B * C; pr += kHeadThreads) {
-    const int b = pr / C, c = pr - b * C;
+  constexpr int kTurn = kHeadThreads / kHeadMaxC;               // samples per turn
+  float zv[64 / kTurn];
+#pragma unroll
+  for (int i = 0; i < 64 / kTurn; ++i) {
+    const int b = i * kTurn + (t >> 4), c = t & (kHeadMaxC - 1);
+    zv[i] = -INFINITY;
+    if (b >= B || c >= C) continue;
     float v[kHeadClusterMax];
 #pragma unroll
     for (int r = 0; r < kHeadClusterMax; ++r)
@@ -157,15 +185,16 @@ __device__ __forceinline__ void head_body(const HeadArgs& a, uint8_t* smem, int 
 #pragma unroll
     for (int r = 0; r < kHeadClusterMax; ++r)
       if (r < S) z = __fadd_rn(z, v[r]);
-    zz[b * kHeadMaxC + c] = __fadd_rn(z, bls[c]);
+    zv[i] = __fadd_rn(z, bls[c]);
   }
-  cluster_sync();   // every CTA is done with the partials
-  // Softmax cross-entropy: 16 lanes per sample (one per class slot), max and sum of
-  // exponentials by butterflies over the sample's lanes.
-  for (int b0 = 0; b0 < Bn; b0 += kHeadThreads / kHeadMaxC) {
-    const int b = b0 + (t >> 4), c = t & (kHeadMaxC - 1);
+  __syncwarp();
+  cluster_arrive();   // this thread is done with the partials; the wait is at the end
+#pragma unroll
+  for (int i = 0; i < 64 / kTurn; ++i) {
+    if (i * kTurn >= Bn) break;
+    const int b = i * kTurn + (t >> 4), c = t & (kHeadMaxC - 1);
     const bool live = b < B && c < C;
-    const float z = live ? zz[b * kHeadMaxC + c] : -INFINITY;
+    const float z = zv[i];
     float m = z;
 #pragma unroll
     for (int off = 1; off < kHeadMaxC; off <<= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
@@ -190,31 +219,19 @@ __device__ __forceinline__ void head_body(const HeadArgs& a, uint8_t* smem, int 
   if (s == 0) {
     if (t < C) {
       float db = 0.f;
+#pragma unroll 8
       for (int b = 0; b < B; ++b) db = __fadd_rn(db, gs[b * kHeadMaxC + t]);
       bL[t] = __fsub_rn(bls[t], __fmul_rn(a.lr, db));
     } else if (t == 32) {
       float l = 0.f;
+#pragma unroll 8
       for (int b = 0; b < B; ++b) l += rl[b];
       a.loss[j] = l / B;
     }
   }
 
-  // ---- 3. backward of the slice: one 8-feature column block per warp at a time.
-  // The fp32 values this lane updates are loaded first; the MMAs hide their latency.
-  auto load_upd = [&](int nt, float2 (&w32)[2], float2& bp32) {
-    const int f = nt * 8 + (lane & 3) * 2;
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int c = (lane >> 2) + 8 * h;
-      w32[h] = c < C ? *reinterpret_cast<const float2*>(Wr + static_cast<int64_t>(c) * in + k0 + f)
-                     : make_float2(0.f, 0.f);
-    }
-    bp32 = (a.has_dx && lane < 4)
-               ? *reinterpret_cast<const float2*>(a.bias_prev_src + src_row + k0 + f)
-               : make_float2(0.f, 0.f);
-  };
-  float2 nw32[2], nbp32;
-  if (warp < kc / 8) load_upd(warp, nw32, nbp32);
+  // ---- 3. backward of the slice: one 8-feature column block per warp at a time, the next
+  // block's fp32 values loaded ahead.
   for (int nt = warp; nt < kc / 8; nt += kHeadThreads / 32) {
     const int f = nt * 8 + (lane & 3) * 2;                      // this lane's two features
     float2 w32[2] = {nw32[0], nw32[1]}, bp32 = nbp32;
@@ -273,6 +290,8 @@ __device__ __forceinline__ void head_body(const HeadArgs& a, uint8_t* smem, int 
                         __fsub_rn(w32[h].y, __fmul_rn(a.lr, dw[2 * h + 1])));
     }
   }
+  __syncwarp();
+  cluster_wait();     // every rank has read this CTA's partials: it may exit
 }
 
 }  // namespace head
