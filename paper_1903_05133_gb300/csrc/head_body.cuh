@@ -36,12 +36,6 @@ __device__ __forceinline__ void cluster_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;"
                ::: "memory");
 }
-__device__ __forceinline__ void cluster_arrive() {
-  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void cluster_wait() {
-  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
 // The float at the same shared-memory offset in CTA `rank` of this cluster.
 __device__ __forceinline__ float ld_cluster(const float* p, int rank) {
   const uint32_t la = static_cast<uint32_t>(__cvta_generic_to_shared(p));

@@ -371,7 +371,7 @@ __global__ void __launch_bounds__(kT, 2) k_small(const SmallArgs a) {
           if (kBf16) *reinterpret_cast<float4*>(part + b * F + 4 * q) = v;   // unrounded, for the bias
         }
         __syncwarp();
-        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+        cluster_arrive();
         __syncthreads();
         for (int n = t; n < F; n += kT) {
           const float* src = kBf16 ? part : own;
@@ -408,7 +408,7 @@ __global__ void __launch_bounds__(kT, 2) k_small(const SmallArgs a) {
       }
       __syncthreads();                  // dZ_{l+1} has been read
       if (l > 0) {
-        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+        cluster_wait();
         const int op1 = kR * F;
         const Div dc(kR * q4);
         for (int idx = t; idx < B * kR * q4; idx += kT) {
