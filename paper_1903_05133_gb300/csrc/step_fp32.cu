@@ -742,20 +742,28 @@ __global__ void __launch_bounds__(kThreads) k_head_f32(const Head32Args a) {
     // cluster barrier per step: zp alternates, and a rank writes it again only after the
     // next step's barrier, which follows every rank's reads here.
     cluster_sync_all();
-    for (int e = t; e < (B + 15) / 16 * 16 * kHeadC; e += kThreads) {
-      const int b = e >> 4, c = e & 15;
+    float zv[kHeadB * kHeadC / kThreads];          // every turn's remote loads in flight
+#pragma unroll
+    for (int i = 0; i < kHeadB * kHeadC / kThreads; ++i) {
+      const int e = t + i * kThreads, b = e >> 4, c = e & 15;
+      zv[i] = 0.f;
+      if (b >= B || c >= C) continue;
+      float v[kHeadSplit];
+#pragma unroll
+      for (int r = 0; r < kHeadSplit; ++r) v[r] = r < S ? ld_cluster_f1(zp + e, r) : 0.f;
+      float z = v[0];
+#pragma unroll
+      for (int r = 1; r < kHeadSplit; ++r)
+        if (r < S) z = __fadd_rn(z, v[r]);
+      zv[i] = __fadd_rn(z, bls[c]);
+    }
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < kHeadB * kHeadC / kThreads; ++i) {
+      const int e = t + i * kThreads, b = e >> 4, c = e & 15;
+      if (i * kThreads / kHeadC >= B) break;
       const bool live = b < B && c < C;
-      float z = 0.f;
-      if (live) {
-        float v[kHeadSplit];
-#pragma unroll
-        for (int r = 0; r < kHeadSplit; ++r) v[r] = r < S ? ld_cluster_f1(zp + e, r) : 0.f;
-        z = v[0];
-#pragma unroll
-        for (int r = 1; r < kHeadSplit; ++r)
-          if (r < S) z = __fadd_rn(z, v[r]);
-        z = __fadd_rn(z, bls[c]);
-      }
+      const float z = zv[i];
       float m = live ? z : -INFINITY;
 #pragma unroll
       for (int off = 1; off < kHeadC; off <<= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
@@ -840,14 +848,17 @@ __global__ void __launch_bounds__(kThreads) k_head_f32(const Head32Args a) {
         }
       }
     }
-    // every rank keeps b_L; rank 0 writes it and the loss
-    if (t < C) {
+    // every rank keeps b_L; rank 0 writes it and the loss (the last warp, which has no weights
+    // to update where slices are narrow)
+    if (t >= kThreads - 32 && lane < C) {
       float db = 0.f;
-      for (int b = 0; b < B; ++b) db = __fadd_rn(db, g[b * kHeadC + t]);
-      bls[t] = __fsub_rn(bls[t], __fmul_rn(a.lr, db));
-      if (last && s == 0) a.bias[j * a.ld + t] = bls[t];
-    } else if (last && s == 0 && t == 32) {
+#pragma unroll 8
+      for (int b = 0; b < B; ++b) db = __fadd_rn(db, g[b * kHeadC + lane]);
+      bls[lane] = __fsub_rn(bls[lane], __fmul_rn(a.lr, db));
+      if (last && s == 0) a.bias[j * a.ld + lane] = bls[lane];
+    } else if (last && s == 0 && t == kThreads - 1) {
       float l = 0.f;
+#pragma unroll 8
       for (int b = 0; b < B; ++b) l += rl[b];
       a.loss[j] = l / B;
     }
