@@ -13,8 +13,10 @@
 // latency (barriers, phases of under a microsecond on 8 of the SMs per learner); products run
 // as FFMA on 4 x 4 outputs per thread.  bf16 operands are rounded to bf16 values held in fp32,
 // whose products are exact in fp32.
-// (264-136-200-13, P = 6, B = 20: 20 us per step of a round, 29 by step(); 12 phases and 5 cluster
-// barriers; 512 threads instead of 256 took as long.)
+// (264-136-200-13, P = 6, B = 20: 19 us per step of a round, 23 by step(), 5 cluster barriers and
+// some 15 phases of 1000 to 5000 cycles; 512 threads instead of 256 took as long.  The weights
+// come by cp.async, all layers in flight, and leave from the last update: 29 us by step() with
+// plain loads, a pass of its own for the stores and dZ rows on the same banks.)
 #include <cstdint>
 #include <type_traits>
 #include <cuda_bf16.h>
@@ -57,7 +59,7 @@ SmallLayout small_layout(const int* dims, int L, int B, bool bf16) {
   }
   s.z[0] = take(B4 * s.wide);
   s.z[1] = take(B4 * s.wide);
-  s.dz = take(B4 * s.wide);
+  s.dz = take(B4 * (s.wide + 4));
   s.own[0] = take(B4 * (s.wide / kR));
   s.own[1] = take(B4 * (s.wide / kR));
   s.loss = take(B4);
@@ -93,8 +95,8 @@ struct Div {
   __device__ __forceinline__ int operator()(int i) const { return d == 1 ? i : static_cast<int>(__umulhi(i, m)); }
 };
 
-// Partial products z[b][n] = sum_f h[b][f] w[n][f] of a slice: 4 samples x 4 outputs (n, n + no,
-// n + 2 no, n + 3 no) per KS neighbouring lanes, which take every KS-th quad of features and
+// Partial products z[b][n] = sum_f h[b][f] w[n][f] of a slice: 4 samples (b, b + nb, ...) x 4 outputs
+// (n, n + no, ...), so that neighbouring lanes' rows fall on distinct banks, per KS neighbouring lanes, which take every KS-th quad of features and
 // then share out the 16 sums.
 template <int KS>
 __device__ __forceinline__ void forward_slice(const float* h, const float* w, float* z, int F, int p, int op,
@@ -110,12 +112,12 @@ __device__ __forceinline__ void forward_slice(const float* h, const float* w, fl
     const float* wr[4];
 #pragma unroll
     for (int e = 0; e < 4; ++e) wr[e] = w + (n + e * no < out ? n + e * no : n) * p;
-    const float* hr = h + 4 * bb * p;
+    const float* hr = h + bb * p;
 #pragma unroll 2
     for (int f = 4 * part; f < F; f += 4 * KS) {
       float4 hv[4], wv[4];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) hv[i] = *reinterpret_cast<const float4*>(hr + i * p + f);
+      for (int i = 0; i < 4; ++i) hv[i] = *reinterpret_cast<const float4*>(hr + i * nb * p + f);
 #pragma unroll
       for (int e = 0; e < 4; ++e) wv[e] = *reinterpret_cast<const float4*>(wr[e] + f);
 #pragma unroll
@@ -137,7 +139,7 @@ __device__ __forceinline__ void forward_slice(const float* h, const float* w, fl
 #pragma unroll
     for (int k = 0; k < 16 / KS; ++k) {
       const int v = part * (16 / KS) + k, i = v >> 2, c = n + (v & 3) * no;
-      if (c < out) z[(4 * bb + i) * op + c] = acc[k];
+      if (c < out) z[(bb + i * nb) * op + c] = acc[k];
     }
   }
 }
@@ -194,26 +196,24 @@ __global__ void __launch_bounds__(kT, 2) k_small(const SmallArgs a) {
   for (int l = 0; l < L; ++l) {
     const int F = slice(a.dims[l]), p = pitch(F), in = a.dims[l], out = a.dims[l + 1], k0 = s * F;
     const float* W = P + a.woff[l] + k0;
-    auto put = [&](int at, float4 v) {
-      *reinterpret_cast<float4*>(sm + o.w[l] + at) = v;
-      if constexpr (kBf16) *reinterpret_cast<float4*>(sm + o.wq[l] + at) = rnd4<true>(v);
+    auto copy = [&](int at, const float* src, int n, auto bytes) {   // n floats of it, then zeros
+      asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;" ::"r"(smem_u32(sm + o.w[l] + at)),
+                   "l"(n > 0 ? src : P), "n"(decltype(bytes)::value), "r"(4 * n)
+                   : "memory");
     };
-    const Div dq(F / 4);
+    if (in % 4 == 0) {
+      const Div dq(F / 4);
 #pragma unroll 4
-    for (int idx = t; idx < out * (F / 4); idx += kT) {
-      const int r = dq(idx), f = 4 * (idx - r * (F / 4));
-      const float* src = W + static_cast<int64_t>(r) * in + f;
-      const int left = in - k0 - f;
-      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (in % 4 == 0) {
-        if (left > 0) v = *reinterpret_cast<const float4*>(src);
-      } else {
-        if (left > 0) v.x = src[0];
-        if (left > 1) v.y = src[1];
-        if (left > 2) v.z = src[2];
-        if (left > 3) v.w = src[3];
+      for (int idx = t; idx < out * (F / 4); idx += kT) {
+        const int r = dq(idx), f = 4 * (idx - r * (F / 4));
+        copy(r * p + f, W + r * in + f, k0 + f < in ? 4 : 0, std::integral_constant<int, 16>{});
       }
-      put(r * p + f, v);
+    } else {
+      const Div df(F);
+      for (int idx = t; idx < out * F; idx += kT) {
+        const int r = df(idx), f = idx - r * F;
+        copy(r * p + f, W + r * in + f, k0 + f < in ? 1 : 0, std::integral_constant<int, 4>{});
+      }
     }
     const float* bias = P + a.boff[l];
     if (l + 1 < L) {
@@ -224,10 +224,20 @@ __global__ void __launch_bounds__(kT, 2) k_small(const SmallArgs a) {
     }
   }
 
+  asm volatile("cp.async.commit_group;" ::: "memory");
+
   int ph = 0;                           // which z buffer the next forward phase writes
   for (int step = 0; step < a.steps; ++step) {
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     __syncthreads();
+    if (kBf16 && step == 0) {           // the weights have arrived too
+      for (int l = 0; l < L; ++l) {
+        const int q = pitch(slice(a.dims[l])) / 4 * a.dims[l + 1];
+        for (int idx = t; idx < q; idx += kT)
+          reinterpret_cast<float4*>(sm + o.wq[l])[idx] =
+              rnd4<true>(reinterpret_cast<const float4*>(sm + o.w[l])[idx]);
+      }
+    }
     {
       const int F = slice(a.dims[0]), p = pitch(F);
       const Div dq(F / 4);
@@ -283,20 +293,28 @@ __global__ void __launch_bounds__(kT, 2) k_small(const SmallArgs a) {
         }
         __syncthreads();
       } else {
-        // logits and cross-entropy, kSmallC lanes per sample
-        for (int e = t; e < (B * kSmallC + kT - 1) / kT * kT; e += kT) {
-          const int b = e / kSmallC, c = e % kSmallC;
+        // logits and cross-entropy, kSmallC lanes per sample, every turn's remote loads in flight
+        constexpr int kTurn = kT / kSmallC;
+        float zv[64 / kTurn];
+#pragma unroll
+        for (int i = 0; i < 64 / kTurn; ++i) {
+          const int b = i * kTurn + t / kSmallC, c = t % kSmallC;
+          zv[i] = 0.f;
+          if (b >= B || c >= C) continue;
+          float v[kR];
+#pragma unroll
+          for (int r = 0; r < kR; ++r) v[r] = ld_cluster_f1(z + b * op + c, r);
+#pragma unroll
+          for (int r = 1; r < kR; ++r) v[0] = __fadd_rn(v[0], v[r]);
+          zv[i] = __fadd_rn(v[0], sm[o.bias[l] + c]);
+        }
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < 64 / kTurn; ++i) {
+          if (i * kTurn >= B) break;
+          const int b = i * kTurn + t / kSmallC, c = t % kSmallC;
           const bool live = b < B && c < C;
-          float x = 0.f;
-          if (live) {
-            float v[kR];
-#pragma unroll
-            for (int r = 0; r < kR; ++r) v[r] = ld_cluster_f1(z + b * op + c, r);
-            x = v[0];
-#pragma unroll
-            for (int r = 1; r < kR; ++r) x = __fadd_rn(x, v[r]);
-            x = __fadd_rn(x, sm[o.bias[l] + c]);
-          }
+          const float x = zv[i];
           float m = live ? x : -INFINITY;
 #pragma unroll
           for (int off = 1; off < kSmallC; off <<= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
@@ -307,7 +325,7 @@ __global__ void __launch_bounds__(kT, 2) k_small(const SmallArgs a) {
           if (live) {
             const float g = __fdiv_rn(__fsub_rn(__fdiv_rn(ex, sum), c == yb[b] ? 1.f : 0.f), static_cast<float>(B));
             if (c == yb[b]) rl[b] = logf(sum) + m - x;
-            dzg[b * op + c] = rnd<kBf16>(g);
+            dzg[b * (op + 4) + c] = rnd<kBf16>(g);
             sm[o.z[ph ^ 1] + b * op + c] = g;     // (free: read before this phase's barrier)
           }
         }
@@ -328,12 +346,13 @@ __global__ void __launch_bounds__(kT, 2) k_small(const SmallArgs a) {
     // ---------------------------------------------------------------- backward
     for (int l = L - 1; l >= 0; --l) {
       const int F = slice(a.dims[l]), p = pitch(F), out = a.dims[l + 1], q4 = F / 4;
-      const int op = kR * slice(out);
+      const int dp = kR * slice(out) + 4;       // pitch of dZ: rows on distinct bank groups
       const float* h = sm + o.h[l];
       const Div dq(q4);
       float* own = sm + o.own[l & 1];
       if (l > 0) {
-        // dZ_l of the own neurons: tiles of 4 samples x 4 neurons, the sum over the outputs
+        // dZ_l of the own neurons: tiles of 4 samples (b, b + nb, ...) x 4
+        // neurons, the sum over the outputs
         // split over ng groups of threads whose partials meet in the free z buffer
         const float* w = sm + o.wq[l];
         float* part = sm + o.z[ph];
@@ -347,21 +366,22 @@ __global__ void __launch_bounds__(kT, 2) k_small(const SmallArgs a) {
           const int g = dt(id), tile = id - g * tiles, bb = dq(tile), q = tile - bb * q4;
           const int o1 = (g + 1) * per < out ? (g + 1) * per : out;
           float4 acc[4] = {};
-          const float* d = dzg + 4 * bb * op;
+          const float* d = dzg + bb * dp;
 #pragma unroll 4
           for (int r = g * per; r < o1; ++r) {
             const float4 wv = *reinterpret_cast<const float4*>(w + r * p + 4 * q);
 #pragma unroll
-            for (int i = 0; i < 4; ++i) acc[i] = fma4(d[i * op + r], wv, acc[i]);
+            for (int i = 0; i < 4; ++i) acc[i] = fma4(d[i * nb * dp + r], wv, acc[i]);
           }
 #pragma unroll
           for (int i = 0; i < 4; ++i)
-            *reinterpret_cast<float4*>(part + ((g * B4) + 4 * bb + i) * F + 4 * q) = acc[i];
+            *reinterpret_cast<float4*>(part + (g * B4 + bb + i * nb) * F + 4 * q) = acc[i];
         }
         __syncthreads();
         for (int idx = t; idx < B * q4; idx += kT) {
           const int b = dq(idx), q = idx - b * q4;
           float4 v = *reinterpret_cast<const float4*>(part + b * F + 4 * q);
+#pragma unroll 4
           for (int g = 1; g < ng; ++g)
             v = add4(v, *reinterpret_cast<const float4*>(part + (g * B4 + b) * F + 4 * q));
           const float4 hv = *reinterpret_cast<const float4*>(h + b * p + 4 * q);
@@ -381,14 +401,17 @@ __global__ void __launch_bounds__(kT, 2) k_small(const SmallArgs a) {
           sm[o.bias[l - 1] + n] = upd(sm[o.bias[l - 1] + n], a.lr, db);
         }
       }
-      // W_l of the own columns: 4 outputs x 4 inputs per thread, samples in ascending order
+      // W_l of the own columns: 4 outputs x 4 inputs per thread, samples in ascending order; the
+      // last step writes it out
+      const int in = a.dims[l], k0 = s * F;
+      const bool last = step + 1 == a.steps;
       const int no = (out + 3) / 4;
       for (int id = t; id < no * q4; id += kT) {
         const int n = dq(id), q = id - n * q4;
         float4 acc[4] = {};
 #pragma unroll 4
         for (int b = 0; b < B; ++b) {
-          const float4 d = *reinterpret_cast<const float4*>(dzg + b * op + 4 * n);
+          const float4 d = *reinterpret_cast<const float4*>(dzg + b * dp + 4 * n);
           const float4 hv = *reinterpret_cast<const float4*>(h + b * p + 4 * q);
           acc[0] = fma4(d.x, hv, acc[0]);
           acc[1] = fma4(d.y, hv, acc[1]);
@@ -402,18 +425,31 @@ __global__ void __launch_bounds__(kT, 2) k_small(const SmallArgs a) {
           float4 w = *reinterpret_cast<const float4*>(sm + o.w[l] + at);
           w = make_float4(upd(w.x, a.lr, acc[e].x), upd(w.y, a.lr, acc[e].y), upd(w.z, a.lr, acc[e].z),
                           upd(w.w, a.lr, acc[e].w));
-          *reinterpret_cast<float4*>(sm + o.w[l] + at) = w;
-          if constexpr (kBf16) *reinterpret_cast<float4*>(sm + o.wq[l] + at) = rnd4<true>(w);
+          if (!last) {
+            *reinterpret_cast<float4*>(sm + o.w[l] + at) = w;
+            if constexpr (kBf16) *reinterpret_cast<float4*>(sm + o.wq[l] + at) = rnd4<true>(w);
+            continue;
+          }
+          const int left = in - k0 - 4 * q;
+          float* dst = P + a.woff[l] + (4 * n + e) * in + k0 + 4 * q;
+          if (in % 4 == 0) {
+            if (left > 0) *reinterpret_cast<float4*>(dst) = w;
+          } else {
+            if (left > 0) dst[0] = w.x;
+            if (left > 1) dst[1] = w.y;
+            if (left > 2) dst[2] = w.z;
+            if (left > 3) dst[3] = w.w;
+          }
         }
       }
       __syncthreads();                  // dZ_{l+1} has been read
       if (l > 0) {
         cluster_wait();
-        const int op1 = kR * F;
+        const int dp1 = kR * F + 4;
         const Div dc(kR * q4);
         for (int idx = t; idx < B * kR * q4; idx += kT) {
           const int b = dc(idx), c = idx - b * kR * q4, r = dq(c), q = c - r * q4;
-          *reinterpret_cast<float4*>(dzg + b * op1 + 4 * c) = ld_cluster_f4(own + b * F + 4 * q, r);
+          *reinterpret_cast<float4*>(dzg + b * dp1 + 4 * c) = ld_cluster_f4(own + b * F + 4 * q, r);
         }
         __syncthreads();
       }
@@ -421,13 +457,7 @@ __global__ void __launch_bounds__(kT, 2) k_small(const SmallArgs a) {
   }
 
   for (int l = 0; l < L; ++l) {
-    const int F = slice(a.dims[l]), p = pitch(F), in = a.dims[l], out = a.dims[l + 1], k0 = s * F;
-    float* W = P + a.woff[l];
-    const Div df(F);
-    for (int idx = t; idx < out * F; idx += kT) {
-      const int r = df(idx), f = idx - r * F;
-      if (k0 + f < in) W[static_cast<int64_t>(r) * in + k0 + f] = sm[o.w[l] + r * p + f];
-    }
+    const int out = a.dims[l + 1];
     float* bias = P + a.boff[l];
     if (l + 1 < L) {
       const int Fo = slice(out);
@@ -446,9 +476,9 @@ __global__ void __launch_bounds__(kT, 2) k_small(const SmallArgs a) {
 // Nets that take these steps.  One wave of clusters: 15 of one CTA per SM, 19 where two fit an
 // SM (784-32-10 bf16, B = 64, a round of 8 steps: P = 16 366 -> 200 us, P = 64 209 -> 466).  Up
 // to 2 M multiply-adds per learner and forward, where the products of eight SMs begin to
-// outweigh the launches saved (784-40-10 bf16, P = 2, B = 64, just below: 213 -> 175 us;
-// 264-136-200-13, P = 6, B = 20, 1.3 M: 145 -> 92 us for 4 steps; fp32 100-37-10, P = 4, B = 7:
-// 49 -> 39 us; 512-96-80-10, P = 2, B = 32, 1.8 M, 8 steps: 271 -> 174 us).  One layer of up to
+// outweigh the launches saved (784-40-10 bf16, P = 2, B = 64, just below: 213 -> 169 us;
+// 264-136-200-13, P = 6, B = 20, 1.3 M: 145 -> 85 us for 4 steps; fp32 100-37-10, P = 4, B = 7:
+// 49 -> 38 us; 512-96-80-10, P = 2, B = 32, 1.8 M, 8 steps: 271 -> 162 us).  One layer of up to
 // 16 classes stays with the head kernels (784-10 bf16, P = 16, B = 64, 28 steps: 308 against
 // 388 us here).
 constexpr int kSmallSms = 152;           // of a GB300
