@@ -2700,13 +2700,12 @@ __global__ void __launch_bounds__(kXentThreads, 1) k_xent_bf16(const float* __re
 // dZ = (p - onehot(y_b)) / B in fp32, a thread per class and sample, its bf16 copy, and
 // b_L -= lr * sum_b dZ (in sample order).  Rank 0 also writes the learner's mean loss.  Bound by
 // the exponentials, divisions and dependent loads of a sample, which one CTA keeps on one SM
-// (P = 32: 1000 classes, B = 32 22.9 -> 12.9 us per launch, 300 classes, B = 16 7.7 -> 7.2;
-// P = 2, 400 classes, B = 64: 3 steps 286 -> 265 us).  With many learners and few logits the
-// SMs are busy as it is, and the cluster's barrier costs more (P = 64, 348 classes, B = 16: a
-// round of 18 steps 356.3 -> 358.8 us).
+// (P = 32, 1000 classes, B = 32: 22.9 -> 12.9 us per launch; P = 2, 400 classes, B = 64: 3 steps
+// 286 -> 265 us).  Below about 12 K logits per learner the cluster's launch and barrier cost what
+// it saves or more (P = 32, 300 classes, B = 16: 7.7 against 7.2 us per launch; P = 2, 622
+// classes, B = 16: 7.9 against 8.2; P = 64, 348, B = 16: a round of 18 steps 356.3 against 358.8).
 constexpr int kXentcThreads = 256, kXentRanks = 8, kXentTile = 128;
-constexpr int kXentSpread = 12288;               // logits per learner from which on it pays for any P ...
-constexpr int kXentSpreadP = 48;                 // ... and learners up to which it pays for any size
+constexpr int kXentSpread = 12288;               // logits per learner
 __global__ void __launch_bounds__(kXentcThreads) k_xent_bf16_cluster(const float* __restrict__ Z,
                                                            const int32_t* __restrict__ y,
                                                            int64_t N, int64_t row0, int B, int Bn,
@@ -2942,7 +2941,7 @@ cudaError_t launch_xent_bf16(const float* Z, const int32_t* y, int64_t N, int64_
                              int Bn, int C, int pitch_c, float lr, const float* bias_src,
                              int src_div, float* bias_L, int64_t ld, __nv_bfloat16* dZ,
                              float* loss, int P, cudaStream_t s) {
-  if (P <= kXentSpreadP || static_cast<int64_t>(B) * C >= kXentSpread)
+  if (static_cast<int64_t>(B) * C >= kXentSpread)
     return launch_pdl(k_xent_bf16_cluster, dim3(kXentRanks, P), dim3(kXentcThreads), 0, s, false, kXentRanks, Z, y,
                       N, row0, B, Bn, C, pitch_c, lr, bias_src, src_div, bias_L, ld, dZ, loss);
   dim3 grid(P, (C + kXentThreads - 1) / kXentThreads);

@@ -762,6 +762,7 @@ def test_small_net_steps(w):
     test_free_global_interval_literal_sequence(w, 2 * w.K1 + 1)
     test_literal_sequence_equals_round(w)
     test_round_host_matches_device_round(w, 0)
+    test_round_host_copies_every_row_it_reads(w, 2 * w.K1 + 1)
 
 
 # The group-sum and head cases above on nets past the one-launch steps' size, so that quads,
@@ -777,15 +778,15 @@ def test_group_sums_past_small_nets(w):
 
 
 # The cross-entropy over a cluster: fewer samples than its CTAs, a last CTA with fewer than
-# the others, more samples than threads, just past and just below the logits from which on the
-# fp32 path spreads it; classes just past the fused epilogue's 128, class slices of more than one
-# tile of 128 with an odd rest, and more learners than take the cluster.
+# the others, more samples than threads, just past and just below the logits from which on it is
+# spread (12288), class slices of one partial tile and of more than one tile of 128 with an odd rest.
 # (300 samples: the mean gradient is small, and the update's bound of 1e-5 has to hold over half
 # an ulp of a weight of 0.6, 3e-8: at lr = 0.05 that is 1.2e-5 of the update, at 1 6e-7.)
 XENT_CASES = [_fp32((40, 36, 1500), 2, 1, 9), _fp32((64, 65), 2, 1, 300).replace(lr=1.0),
               _fp32((40, 33), 3, 1, 373).replace(lr=1.0), _fp32((40, 33), 3, 1, 372).replace(lr=1.0),
-              _small((64, 136, 131), "bf16", 2, 2, 5, 2, 20), _small((64, 72, 1100), "bf16", 3, 1, 64, 2, 130),
-              _small((72, 2056), "bf16", 2, 1, 33, 1, 50), _small((64, 136, 131), "bf16", 50, 2, 5, 2, 20)]
+              _small((64, 72, 2459), "bf16", 2, 2, 5, 2, 20), _small((64, 72, 1100), "bf16", 3, 1, 64, 2, 130),
+              _small((72, 2056), "bf16", 2, 1, 33, 1, 50), _small((64, 136, 193), "bf16", 2, 2, 64, 2, 130),
+              _small((64, 136, 191), "bf16", 2, 2, 64, 2, 130)]
 
 
 @pytest.mark.parametrize("w", XENT_CASES, ids=lambda w: w.name)
