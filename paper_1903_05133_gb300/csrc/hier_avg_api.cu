@@ -25,6 +25,8 @@ using ha::TcFwdArgs;
 constexpr int64_t kAlign = 1024;
 constexpr int64_t kTargetCtas = 152;   // persistent kernels: one CTA per SM of a GB300
 constexpr int64_t kPieceChunks = 48;   // chunks per piece of a split tile (forward, backward)
+constexpr int64_t kFineChunks = 4;     // ... of a backward tile where few tiles leave SMs idle
+constexpr int64_t kStaticScratchBytes = int64_t(32) << 20;   // 32 MiB: step_static's scratch
 int64_t round_up(int64_t x, int64_t m) { return (x + m - 1) / m * m; }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*,
@@ -87,7 +89,7 @@ struct hier_avg {
   std::vector<int> fwd_pc;                    // per layer (dynamic): chunks per tail piece
   int fwd_group = 1;                          // learners per grouped forward after an average
   std::vector<int> bwd_ctas, bwd_tiles;       // per layer: CTAs, input slices of 128
-  std::vector<int> bwd_whole, bwd_np;         // per layer: whole tiles, tail pieces
+  std::vector<int> bwd_whole, bwd_np, bwd_pc; // per layer: whole tiles, tail pieces, chunks per piece
   bool fused_xent = false;                    // d_L <= 128: CE in the last forward epilogue
   bool w_stream = true;                       // parameters exceed L2: stream W evict-first
   bool small = false;                         // whole steps in one launch (either precision)
@@ -178,7 +180,8 @@ namespace {
 
 bool valid_handle(const hier_avg* h) { return h != nullptr; }
 
-int plan_layout(hier_avg* h) {
+// fine: backward tiles of few-tile layers in pieces of kFineChunks.
+void plan_layout(hier_avg* h, bool fine = true) {
   const int L = h->L;
   int64_t pos = 0;
   h->woff.assign(L, 0);
@@ -196,6 +199,7 @@ int plan_layout(hier_avg* h) {
 
   const int64_t P = h->P, B = h->B;
   int64_t off = 0;
+  bool fine_used = false;
   auto take = [&](int64_t bytes) {
     const int64_t o = off;
     off = round_up(off + bytes, kAlign);
@@ -224,6 +228,7 @@ int plan_layout(hier_avg* h) {
     h->bwd_tiles.assign(L, 1);
     h->bwd_whole.assign(L, 0);
     h->bwd_np.assign(L, 1);
+    h->bwd_pc.assign(L, static_cast<int>(kPieceChunks));
     int64_t part_bytes = 16, max_tiles = 1;
     for (int l = 0; l < L; ++l) {
       const int64_t in = h->dims[l], out = h->dims[l + 1];
@@ -268,7 +273,23 @@ int plan_layout(hier_avg* h) {
         // backward 357 -> 361 us per launch.)
         const int64_t nc = (out + 63) / 64;
         const int64_t t_tail = std::min<int64_t>(btiles * P, kTargetCtas);
-        const int64_t np = (nc + kPieceChunks - 1) / kPieceChunks;
+        // Few long tiles (at most kPieceChunks chunks, so whole tiles otherwise) in pieces of
+        // one promotion segment, kFineChunks chunks, while every piece has an SM of its own.
+        // The partials are the segment sums that a whole tile adds in the same order, so dX
+        // keeps its bits.  The partials' round trip costs about 12 chunks' time (B <= 32; more
+        // for larger batches): P = 2, a round of 6 steps of 784-512-n-10, B = 32: n = 512
+        // (8 chunks) 456 -> 464 us, 1000 (16) 416 -> 419, 1200 (19) 570 -> 517, 1536 (24) 545 ->
+        // 432, 2504 (40) 603 -> 500; B = 64: 1200 703 -> 723, 1536 680 -> 625.  Pieces in two
+        // turns lost as often as they won (P = 4, B = 48, 2512: 786 -> 803; P = 8, B = 32, 2048:
+        // 630 -> 528).
+        int64_t pc = kPieceChunks;
+        const int64_t fp = (nc + kFineChunks - 1) / kFineChunks;
+        if (fine && l > 0 && nc <= kPieceChunks && nc >= (h->Bn <= 32 ? 17 : 24) && btiles * P * fp <= kTargetCtas) {
+          pc = kFineChunks;
+          fine_used = true;
+        }
+        h->bwd_pc[l] = static_cast<int>(pc);
+        const int64_t np = (nc + pc - 1) / pc;
         h->bwd_whole[l] = static_cast<int>(btiles * P - t_tail);
         h->bwd_np[l] = static_cast<int>(np);
         h->bwd_ctas[l] = static_cast<int>(
@@ -301,10 +322,11 @@ int plan_layout(hier_avg* h) {
   h->off_Z = take(P * B * h->dims[L] * 4);
   h->off_loss = take(P * 4);
   h->off_err = take(16);
+  // (a step that fits the static scratch without the pieces' partials has to fit it with them)
+  if (fine_used && off > kStaticScratchBytes) return plan_layout(h, false);
   h->ws_step_bytes = off;
   if (h->prec == HA_PREC_BF16 && h->S > 1) h->off_M = take((P / h->S) * h->ld * 4);
   h->ws_bytes = off;
-  return HA_OK;
 }
 
 int make_map(hier_avg* h, CUtensorMap* m, CUtensorMapDataType dt, void* base, uint64_t d0,
@@ -746,7 +768,7 @@ int do_step(hier_avg* h, bool h1_ready = false, bool fuse_next = false, bool* fu
       a.n_tiles = h->bwd_tiles[l] * P;
       a.n_whole = h->bwd_whole[l];
       a.np_tail = h->bwd_np[l];
-      a.piece_chunks = static_cast<int>(kPieceChunks);
+      a.piece_chunks = h->bwd_pc[l];
       a.dyn = h->wsp<int>(h->off_dyn);
       a.part = h->wsp<float>(h->off_part);
       a.counters = h->wsp<int>(h->off_cnt);
@@ -1469,8 +1491,6 @@ int hier_avg_profile_read(hier_avg* h, int kind, double* total_ms, int64_t* laun
 // split-K partial sums and tile counters) lives in this file-scope array instead
 // of a caller workspace.  Every GPU that loads the library holds it until exit.
 namespace {
-
-constexpr int64_t kStaticScratchBytes = int64_t(32) << 20;   // 32 MiB
 
 static __device__ __align__(256) unsigned char g_static_scratch[kStaticScratchBytes];
 

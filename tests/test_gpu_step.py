@@ -777,6 +777,17 @@ def test_group_sums_past_small_nets(w):
     test_literal_sequence_equals_round(w)
 
 
+# The backward of few long tiles in pieces of one promotion segment: a last piece of one chunk,
+# a ragged layer, 48 chunks in 12 pieces (the last length that is not split in pieces of 48), and
+# a class layer whose dX is split.
+@pytest.mark.parametrize("w", [_head((128, 512, 1088, 10), 2, 2, 32, 128), _head((64, 200, 1608, 13), 3, 1, 20, 50),
+                               _head((64, 256, 3072, 10), 2, 1, 64, 256), _head((64, 264, 1500), 4, 2, 16, 64)],
+                         ids=lambda w: w.name)
+def test_backward_in_segment_pieces(w):
+    test_one_step_from_distinct_learners(w)
+    test_literal_sequence_equals_round(w)
+
+
 # The cross-entropy over a cluster: fewer samples than its CTAs, a last CTA with fewer than
 # the others, more samples than threads, just past and just below the logits from which on it is
 # spread (12288), class slices of one partial tile and of more than one tile of 128 with an odd rest.
