@@ -220,7 +220,7 @@ constexpr int kSmallC = 32;       // classes at most
 // rounded to bf16 on the bf16 path), its rows of H_l, and b_l of its neurons.
 struct SmallLayout {
   int w[kSmallLayers], wq[kSmallLayers], h[kSmallLayers], bias[kSmallLayers];
-  int z[2], dz, own[2], loss, labels, raw, total;
+  int z[2], dz, own[2], g, loss, labels, raw, total;
   int wide;                       // outputs of the widest layer, whole slices
 };
 struct SmallArgs {

@@ -13,10 +13,12 @@
 // latency (barriers, phases of under a microsecond on 8 of the SMs per learner); products run
 // as FFMA on 4 x 4 outputs per thread.  bf16 operands are rounded to bf16 values held in fp32,
 // whose products are exact in fp32.
-// (264-136-200-13, P = 6, B = 20: 19 us per step of a round, 23 by step(), 5 cluster barriers and
+// (264-136-200-13, P = 6, B = 20: 18.5 us per step of a round, 22.5 by step(), 5 cluster barriers and
 // some 15 phases of 1000 to 5000 cycles; 512 threads instead of 256 took as long.  The weights
 // come by cp.async, all layers in flight, and leave from the last update: 29 us by step() with
-// plain loads, a pass of its own for the stores and dZ rows on the same banks.)
+// plain loads, a pass of its own for the stores and dZ rows on the same banks.  Up to 16 classes
+// take 16 lanes per sample, and b_L and the loss are the last warp's while the others go on:
+// 784-40-10, B = 64 21 -> 18.5 us per step.)
 #include <cstdint>
 #include <type_traits>
 #include <cuda_bf16.h>
@@ -62,6 +64,7 @@ SmallLayout small_layout(const int* dims, int L, int B, bool bf16) {
   s.dz = take(B4 * (s.wide + 4));
   s.own[0] = take(B4 * (s.wide / kR));
   s.own[1] = take(B4 * (s.wide / kR));
+  s.g = take(B4 * kSmallC);
   s.loss = take(B4);
   s.labels = take(2 * B4);
   s.raw = take(bf16 ? (B * slice(dims[0]) + 1) / 2 : B * slice(dims[0]));
@@ -140,6 +143,47 @@ __device__ __forceinline__ void forward_slice(const float* h, const float* w, fl
     for (int k = 0; k < 16 / KS; ++k) {
       const int v = part * (16 / KS) + k, i = v >> 2, c = n + (v & 3) * no;
       if (c < out) z[(bb + i * nb) * op + c] = acc[k];
+    }
+  }
+}
+
+// Logits (the ranks' partials in order, then b_L) and softmax cross-entropy of the whole batch,
+// LC lanes per sample, every turn's remote loads in flight: dz (rounded), g and the samples' losses.
+template <bool kBf16, int LC>
+__device__ __forceinline__ void cross_entropy(const float* z, int op, const float* bias, const int* y, float* dz,
+                                              float* g, float* loss, int B, int C, int t) {
+  constexpr int kTurn = kT / LC;
+  float zv[64 / kTurn];
+#pragma unroll
+  for (int i = 0; i < 64 / kTurn; ++i) {
+    const int b = i * kTurn + t / LC, c = t % LC;
+    zv[i] = 0.f;
+    if (b >= B || c >= C) continue;
+    float v[kR];
+#pragma unroll
+    for (int r = 0; r < kR; ++r) v[r] = ld_cluster_f1(z + b * op + c, r);
+#pragma unroll
+    for (int r = 1; r < kR; ++r) v[0] = __fadd_rn(v[0], v[r]);
+    zv[i] = __fadd_rn(v[0], bias[c]);
+  }
+  __syncwarp();
+#pragma unroll
+  for (int i = 0; i < 64 / kTurn; ++i) {
+    if (i * kTurn >= B) break;
+    const int b = i * kTurn + t / LC, c = t % LC;
+    const bool live = b < B && c < C;
+    float m = live ? zv[i] : -INFINITY;
+#pragma unroll
+    for (int off = 1; off < LC; off <<= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
+    const float ex = live ? expf(zv[i] - m) : 0.f;
+    float sum = ex;
+#pragma unroll
+    for (int off = 1; off < LC; off <<= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
+    if (live) {
+      const float gv = __fdiv_rn(__fsub_rn(__fdiv_rn(ex, sum), c == y[b] ? 1.f : 0.f), static_cast<float>(B));
+      if (c == y[b]) loss[b] = logf(sum) + m - zv[i];
+      dz[b * (op + 4) + c] = rnd<kBf16>(gv);
+      g[b * kSmallC + c] = gv;
     }
   }
 }
@@ -293,54 +337,25 @@ __global__ void __launch_bounds__(kT, 2) k_small(const SmallArgs a) {
         }
         __syncthreads();
       } else {
-        // logits and cross-entropy, kSmallC lanes per sample, every turn's remote loads in flight
-        constexpr int kTurn = kT / kSmallC;
-        float zv[64 / kTurn];
-#pragma unroll
-        for (int i = 0; i < 64 / kTurn; ++i) {
-          const int b = i * kTurn + t / kSmallC, c = t % kSmallC;
-          zv[i] = 0.f;
-          if (b >= B || c >= C) continue;
-          float v[kR];
-#pragma unroll
-          for (int r = 0; r < kR; ++r) v[r] = ld_cluster_f1(z + b * op + c, r);
-#pragma unroll
-          for (int r = 1; r < kR; ++r) v[0] = __fadd_rn(v[0], v[r]);
-          zv[i] = __fadd_rn(v[0], sm[o.bias[l] + c]);
-        }
-        __syncwarp();
-#pragma unroll
-        for (int i = 0; i < 64 / kTurn; ++i) {
-          if (i * kTurn >= B) break;
-          const int b = i * kTurn + t / kSmallC, c = t % kSmallC;
-          const bool live = b < B && c < C;
-          const float x = zv[i];
-          float m = live ? x : -INFINITY;
-#pragma unroll
-          for (int off = 1; off < kSmallC; off <<= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
-          const float ex = live ? expf(x - m) : 0.f;
-          float sum = ex;
-#pragma unroll
-          for (int off = 1; off < kSmallC; off <<= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
-          if (live) {
-            const float g = __fdiv_rn(__fsub_rn(__fdiv_rn(ex, sum), c == yb[b] ? 1.f : 0.f), static_cast<float>(B));
-            if (c == yb[b]) rl[b] = logf(sum) + m - x;
-            dzg[b * (op + 4) + c] = rnd<kBf16>(g);
-            sm[o.z[ph ^ 1] + b * op + c] = g;     // (free: read before this phase's barrier)
-          }
-        }
+        if (C <= 16)
+          cross_entropy<kBf16, 16>(z, op, sm + o.bias[l], yb, dzg, sm + o.g, rl, B, C, t);
+        else
+          cross_entropy<kBf16, kSmallC>(z, op, sm + o.bias[l], yb, dzg, sm + o.g, rl, B, C, t);
         __syncthreads();
-        if (t < C) {
+        // the last warp adds b_L's gradient and the loss while the others go on
+        if (t >= kT - 32 && t - (kT - 32) < C) {
+          const int c = t - (kT - 32);
           float db = 0.f;
 #pragma unroll 8
-          for (int b = 0; b < B; ++b) db = __fadd_rn(db, sm[o.z[ph ^ 1] + b * op + t]);
-          sm[o.bias[l] + t] = upd(sm[o.bias[l] + t], a.lr, db);
-        } else if (s == 0 && t == kT - 1 && step + 1 == a.steps) {
+          for (int b = 0; b < B; ++b) db = __fadd_rn(db, sm[o.g + b * kSmallC + c]);
+          sm[o.bias[l] + c] = upd(sm[o.bias[l] + c], a.lr, db);
+        }
+        if (s == 0 && t == kT - 33 && step + 1 == a.steps) {
           float x = 0.f;
+#pragma unroll 8
           for (int b = 0; b < B; ++b) x += rl[b];
           a.loss[j] = x / B;
         }
-        __syncthreads();
       }
     }
     // ---------------------------------------------------------------- backward
@@ -474,11 +489,11 @@ __global__ void __launch_bounds__(kT, 2) k_small(const SmallArgs a) {
 }  // namespace
 
 // Nets that take these steps.  One wave of clusters: 15 of one CTA per SM, 19 where two fit an
-// SM (784-32-10 bf16, B = 64, a round of 8 steps: P = 16 366 -> 200 us, P = 64 209 -> 466).  Up
+// SM (784-32-10 bf16, B = 64, a round of 8 steps: P = 16 366 -> 182 us, P = 64 209 -> 466).  Up
 // to 2 M multiply-adds per learner and forward, where the products of eight SMs begin to
-// outweigh the launches saved (784-40-10 bf16, P = 2, B = 64, just below: 213 -> 169 us;
-// 264-136-200-13, P = 6, B = 20, 1.3 M: 145 -> 85 us for 4 steps; fp32 100-37-10, P = 4, B = 7:
-// 49 -> 38 us; 512-96-80-10, P = 2, B = 32, 1.8 M, 8 steps: 271 -> 162 us).  One layer of up to
+// outweigh the launches saved (784-40-10 bf16, P = 2, B = 64, just below: 213 -> 148 us;
+// 264-136-200-13, P = 6, B = 20, 1.3 M: 145 -> 82 us for 4 steps; fp32 100-37-10, P = 4, B = 7:
+// 49 -> 37 us; 512-96-80-10, P = 2, B = 32, 1.8 M, 8 steps: 271 -> 151 us).  One layer of up to
 // 16 classes stays with the head kernels (784-10 bf16, P = 16, B = 64, 28 steps: 308 against
 // 388 us here).
 constexpr int kSmallSms = 152;           // of a GB300
