@@ -2,12 +2,13 @@
 // sum of the local SGD step (Algorithm 1 inner loop, Sec. 3.1) stays in fp32 (FFMA;
 // bf16 or tf32 operands are outside this mode's tolerance).
 //
-//   k_fwd_f32   Z = H W^T + b (ReLU)   one tile of 8-64 samples x 64 outputs per CTA
-//   k_dx_f32    dZ' = (dZ W) [H > 0]   the same tile shape over samples x inputs
+//   k_tile_f32<BM, false>  Z = H W^T + b (ReLU)   one tile of 8-64 samples x 64 outputs per CTA
+//   k_tile_f32<BM, true>   dZ' = (dZ W) [H > 0]   the same tile shape over samples x inputs
 //   k_dw_f32    W -= lr dZ^T H, b -= lr sum dZ   64 outputs x 128 inputs per CTA
-//   k_xent_f32  softmax cross-entropy gradient
+//   k_xent_f32, k_xent_f32_cluster               softmax cross-entropy gradient
 //   k_head_f32  the whole last layer (forward, cross-entropy, dX, update) when it has at
 //               most 16 classes; for a one-layer model several local steps per launch
+// (Small nets run whole steps in one launch instead, whichever the precision: step_small.cu.)
 // The first layer reads its batch rows straight from X (no gather).  Rows whose length is a
 // multiple of four floats move as 16-byte cp.async copies, others as 4-byte ones.
 // Rounds against 16 x 16-tile kernels with one output per thread and a serial reduction

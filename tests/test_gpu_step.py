@@ -224,10 +224,9 @@ SMALL_FP32 = configs.Workload("tiny_mlp_fp32", P=4, S=2, K1=2, K2=2, rounds=1,
                               sigma_mu=0.1, init="he")
 
 
-# Last-layer paths: CUDA-core head kernels (<= 16 classes; SMALL_BF16, SOFTMAX_BF16 which
-# reads X directly, the 16-learner MLP, HEAD_C13 with a class count that is not the
-# specialised 10, RAGGED_BF16: 13 classes over a 200-wide ragged input), tensor-core forward
-# with the CE in its epilogue (WIDE_SOFTMAX_BF16),
+# Last-layer paths: the head kernels (<= 16 classes; SMALL_BF16, SOFTMAX_BF16 which reads X
+# directly, the 16-learner MLP), whole steps in one launch (nets as small as HEAD_C13 and
+# RAGGED_BF16), tensor-core forward with the CE in its epilogue (WIDE_SOFTMAX_BF16),
 # and the standalone CE kernel (MANY_CLASSES_BF16: 300 classes over 3 tiles).
 STEP_CASES = [configs.SOFTMAX_P4, SMALL_FP32, SMALL_BF16, SOFTMAX_BF16, HEAD_C13,
               WIDE_SOFTMAX_BF16, RAGGED_BF16, MANY_CLASSES_BF16, configs.MLP512_P16, FUSE_PIECES,
@@ -285,6 +284,8 @@ def test_full_run_against_oracle(w):
 # per cluster); Q = 2 with S = 6 (three per cluster: the generic tree) and a ragged
 # 200-input layer; Q = 4 with S = 12 and K1 = 1 (every step both reads the cluster
 # means and writes group sums); Q = 2 because the batch is 64.
+# (Nets of these sizes run whole steps in one launch; test_group_sums_past_small_nets repeats
+# the cases on wider ones.)
 GROUP_S8 = configs.Workload("mlp_bf16_group4_S8", P=16, S=8, K1=2, K2=3, rounds=1,
                             dims=(256, 192, 10), precision="bf16", N=128, B=32, lr=0.05,
                             sigma_mu=0.1, init="he")
