@@ -414,6 +414,17 @@ int build_maps(hier_avg* h) {
   return HA_OK;
 }
 
+// Attributes of the kernels that the handle's steps launch, and their tensor maps (small nets
+// use none).
+int configure(hier_avg* h) {
+  const char* what = "kernel attributes";
+  if (h->small) return h->cuda(ha::small_configure(), what);
+  if (h->prec != HA_PREC_BF16) return h->cuda(ha::fp32_configure(), what);
+  if (int rc = h->cuda(ha::tc_configure(), what)) return rc;
+  if (int rc = h->cuda(ha::head_configure(), what)) return rc;
+  return build_maps(h);
+}
+
 int check_bound(hier_avg* h) {
   if (!h) return HA_EINVAL;
   if (!h->bound) return h->fail(HA_ESTATE, "hier_avg_bind has not been called");
@@ -1261,16 +1272,7 @@ int hier_avg_bind(hier_avg* h, float* params_dev, void* workspace_dev, int64_t w
     h->upd_group = h->S % 4 == 0 && ha::tc_update_max_group(h->Bn) >= 4 ? 4 : 2;
   int rc;
   if ((rc = h->cuda(cudaMemsetAsync(h->ws, 0, h->ws_step_bytes, h->stream), "bind: memset"))) return rc;
-  if (h->prec == HA_PREC_BF16) {
-    if ((rc = h->cuda(ha::tc_configure(), "bind: kernel attributes"))) return rc;
-    if ((rc = h->cuda(ha::head_configure(), "bind: kernel attributes"))) return rc;
-    if ((rc = h->cuda(ha::small_configure(), "bind: kernel attributes"))) return rc;
-    if ((rc = build_maps(h))) return rc;
-  } else if ((rc = h->cuda(ha::small_configure(), "bind: kernel attributes"))) {
-    return rc;
-  } else if ((rc = h->cuda(ha::fp32_configure(), "bind: kernel attributes"))) {
-    return rc;
-  }
+  if ((rc = configure(h))) return rc;
   h->bound = true;
   return HA_OK;
 }
@@ -1592,16 +1594,7 @@ extern "C" int hier_avg_step_static(hier_avg* h, float* params_dev, const void* 
     return rc;
   h->m_ok = false;   // the array holds a step's scratch only: rounds average in place
   h->upd_group = 1;
-  if (h->prec == HA_PREC_BF16) {
-    if ((rc = h->cuda(ha::tc_configure(), "step_static: kernel attributes"))) return rc;
-    if ((rc = h->cuda(ha::head_configure(), "step_static: kernel attributes"))) return rc;
-    if ((rc = h->cuda(ha::small_configure(), "step_static: kernel attributes"))) return rc;
-    if ((rc = build_maps(h))) return rc;
-  } else if ((rc = h->cuda(ha::small_configure(), "step_static: kernel attributes"))) {
-    return rc;
-  } else if ((rc = h->cuda(ha::fp32_configure(), "step_static: kernel attributes"))) {
-    return rc;
-  }
+  if ((rc = configure(h))) return rc;
   h->bound = true;
   return do_step(h);
 }
