@@ -32,20 +32,6 @@ __device__ __forceinline__ const __nv_bfloat16* head_row(const HeadArgs& a, int 
   return a.H + (static_cast<int64_t>(j) * a.Bn + b) * a.pitch_in;
 }
 
-__device__ __forceinline__ void cluster_sync() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;"
-               ::: "memory");
-}
-// The float at the same shared-memory offset in CTA `rank` of this cluster.
-__device__ __forceinline__ float ld_cluster(const float* p, int rank) {
-  const uint32_t la = static_cast<uint32_t>(__cvta_generic_to_shared(p));
-  uint32_t ra;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(la), "r"(rank));
-  float v;
-  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(ra) : "memory");
-  return v;
-}
-
 // ---- warp-level MMA helpers (m16n8k16, bf16 inputs, fp32 accumulators)
 __device__ __forceinline__ void ldsm_x4(const void* p, uint32_t (&r)[4]) {
   asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
@@ -74,9 +60,6 @@ __device__ __forceinline__ void mma16816(float (&d)[4], const uint32_t (&a)[4], 
 // offset (0 or 8): the four 8x8 matrices are (rows 0-7 | 8-15) x (cols 0-7 | 8-15).
 __device__ __forceinline__ int a_row(int l) { return ((l >> 3) & 1) * 8 + (l & 7); }
 __device__ __forceinline__ int a_col(int l) { return (l >> 4) * 8; }
-
-
-
 
 // Shared memory needed by head_body for slices of F features.
 __host__ __device__ inline int head_body_smem(int F, int Bn) {
@@ -163,7 +146,7 @@ __device__ __forceinline__ void head_body(const HeadArgs& a, uint8_t* smem, int 
   // ---- 2. full logits (partials added in slice order) and softmax cross-entropy: 16 lanes
   // per sample (one per class slot), every sample's remote loads in flight together, max and
   // sum of exponentials by butterflies over the sample's lanes.
-  cluster_sync();
+  cluster_sync_all();
   constexpr int kTurn = kHeadThreads / kHeadMaxC;               // samples per turn
   float zv[64 / kTurn];
 #pragma unroll
@@ -174,14 +157,13 @@ __device__ __forceinline__ void head_body(const HeadArgs& a, uint8_t* smem, int 
     float v[kHeadClusterMax];
 #pragma unroll
     for (int r = 0; r < kHeadClusterMax; ++r)
-      v[r] = r < S ? ld_cluster(zp + b * kHeadMaxC + c, r) : 0.f;
+      v[r] = r < S ? ld_cluster_f1(zp + b * kHeadMaxC + c, r) : 0.f;
     float z = 0.f;
 #pragma unroll
     for (int r = 0; r < kHeadClusterMax; ++r)
       if (r < S) z = __fadd_rn(z, v[r]);
     zv[i] = __fadd_rn(z, bls[c]);
   }
-  __syncwarp();
   cluster_arrive();   // this thread is done with the partials; the wait is at the end
 #pragma unroll
   for (int i = 0; i < 64 / kTurn; ++i) {
@@ -225,8 +207,10 @@ __device__ __forceinline__ void head_body(const HeadArgs& a, uint8_t* smem, int 
   }
 
   // ---- 3. backward of the slice: one 8-feature column block per warp at a time, the next
-  // block's fp32 values loaded ahead.
+  // block's fp32 values loaded ahead.  (ldmatrix and mma.sync are .aligned too: the warp comes
+  // together before those that follow lane-dependent code.)
   for (int nt = warp; nt < kc / 8; nt += kHeadThreads / 32) {
+    __syncwarp();
     const int f = nt * 8 + (lane & 3) * 2;                      // this lane's two features
     float2 w32[2] = {nw32[0], nw32[1]}, bp32 = nbp32;
     if (nt + kHeadThreads / 32 < kc / 8) load_upd(nt + kHeadThreads / 32, nw32, nbp32);  // next block
@@ -243,6 +227,7 @@ __device__ __forceinline__ void head_body(const HeadArgs& a, uint8_t* smem, int 
     uint32_t wb0, wb1;
     ldsm_x2_t(wq + (lane & 15) * FP + nt * 8, wb0, wb1);
     for (int mt = 0; mt < Bn / 16; ++mt) {
+      __syncwarp();
       uint32_t af[4];
       ldsm_x4(gqa + (mt * 16 + a_row(lane)) * kGA + a_col(lane), af);
       float dh[4] = {0.f, 0.f, 0.f, 0.f};
@@ -284,7 +269,6 @@ __device__ __forceinline__ void head_body(const HeadArgs& a, uint8_t* smem, int 
                         __fsub_rn(w32[h].y, __fmul_rn(a.lr, dw[2 * h + 1])));
     }
   }
-  __syncwarp();
   cluster_wait();     // every rank has read this CTA's partials: it may exit
 }
 

@@ -78,17 +78,21 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, int* e
 }
 
 // ------------------------------------------------ thread-block clusters
-// Barrier over every thread of every CTA of the cluster (release / acquire).
-__device__ __forceinline__ void cluster_sync_all() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;"
-               ::: "memory");
-}
-// The same in two halves.
+// Barrier over every thread of every CTA of the cluster (release / acquire).  The .aligned
+// forms have a warp's 32 lanes execute the instruction together, which nothing guarantees
+// after code that took the lanes apart (a loop that is ragged within a warp, a return from an
+// inlined lambda), so each wrapper brings them together first.
 __device__ __forceinline__ void cluster_arrive() {
+  __syncwarp();
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
 }
 __device__ __forceinline__ void cluster_wait() {
+  __syncwarp();
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_sync_all() {
+  cluster_arrive();
+  cluster_wait();
 }
 // The float at the same shared-memory offset in CTA `rank` of this cluster.
 __device__ __forceinline__ float ld_cluster_f1(const float* p, int rank) {

@@ -591,7 +591,6 @@ __global__ void __launch_bounds__(kXentcThreads) k_xent_f32_cluster(const float*
       const float p = __fdiv_rn(expf(Zb[at] - row_max[i]), row_sum[i]);
       d[at] = __fdiv_rn(__fsub_rn(p, row_y[i] == c ? 1.f : 0.f), fB);
     }
-  __syncwarp();
   cluster_wait();                                  // every rank's losses are written
   if (blockIdx.x == 0) {
     float l = 0.f;

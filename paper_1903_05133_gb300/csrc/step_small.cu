@@ -317,7 +317,6 @@ __global__ void __launch_bounds__(kT, 2) k_small(const SmallArgs a) {
       else forward_slice<1>(h, w, z, F, p, op, nb, out, t);
       // One barrier per phase: the buffers alternate, and a rank writes this one again only
       // after the next phase's barrier, which follows every rank's reads here.
-      __syncwarp();
       cluster_sync_all();
       if (l + 1 < L) {
         float* hn = sm + o.h[l + 1];
@@ -405,7 +404,6 @@ __global__ void __launch_bounds__(kT, 2) k_small(const SmallArgs a) {
           *reinterpret_cast<float4*>(own + b * F + 4 * q) = rnd4<kBf16>(v);
           if (kBf16) *reinterpret_cast<float4*>(part + b * F + 4 * q) = v;   // unrounded, for the bias
         }
-        __syncwarp();
         cluster_arrive();
         __syncthreads();
         for (int n = t; n < F; n += kT) {
@@ -482,7 +480,6 @@ __global__ void __launch_bounds__(kT, 2) k_small(const SmallArgs a) {
       for (int n = t; n < out; n += kT) bias[n] = sm[o.bias[l] + n];
     }
   }
-  __syncwarp();
   cluster_sync_all();                   // what the others read here has been read
 }
 

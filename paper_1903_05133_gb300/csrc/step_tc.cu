@@ -2766,7 +2766,6 @@ __global__ void __launch_bounds__(kXentcThreads) k_xent_bf16_cluster(const float
       own_y[i] = yb;
     }
   }
-  __syncwarp();
   cluster_sync_all();
   if (t < B) {
     const int r = t % R, i = t / R;
@@ -2811,7 +2810,6 @@ __global__ void __launch_bounds__(kXentcThreads) k_xent_bf16_cluster(const float
     }
     __syncthreads();
   }
-  __syncwarp();
   cluster_wait();                                  // every rank has read this CTA's statistics
 }
 

@@ -686,7 +686,7 @@ FP32_CASES = [_fp32((64, 64, 17), 4, 2, 8), _fp32((130, 65, 40), 3, 1, 9), _fp32
               _fp32((100, 36, 10), 2, 1, 65), _fp32((2048, 64, 10), 1, 1, 32), _fp32((96, 72, 40), 2, 1, 130),
               _fp32((3072, 10), 2, 2, 64), _fp32((512, 16), 3, 1, 1), _fp32((37, 10), 4, 4, 17),
               _fp32((70, 5), 2, 2, 3), _fp32((8200, 10), 1, 1, 2), _fp32((516, 61, 16), 2, 1, 16),
-              _fp32((516, 61, 16), 2, 1, 31)]
+              _fp32((516, 61, 16), 2, 1, 31), _fp32((2048, 200, 10), 1, 1, 7)]
 
 
 @pytest.mark.parametrize("w", FP32_CASES, ids=lambda w: w.name)
