@@ -56,16 +56,42 @@ __device__ __forceinline__ void store_rows(V* p, int64_t ld_v, int n, V m) {
   for (int i = 0; i < n; ++i) p[static_cast<int64_t>(i) * ld_v] = m;
 }
 
+// Rows whose length is no multiple of four: `tail` = 1 to 3 columns follow the cols_v quads, and
+// the row's last CTA takes them, a thread per column, with the same tree over floats.  (A second
+// launch for them cost 3 to 5 us; the generic kernels, which need none, keep fewer rows in
+// flight.  Rows padded to 64, this | the generic kernels | two launches: P = 16, S = 2, D =
+// 8000001 local + global 150 | 231 | 163 us; P = 64, S = 8, D = 1000003 local 74.8 | 76.8 | 80.0,
+// local + global 87.6 | 121 | 125; P = 128, S = 32, D = 4000001 local + global 618 | 777 | 689.)
+__device__ __forceinline__ bool tail_cta(int tail) { return tail != 0 && blockIdx.x == gridDim.x - 1; }
+__device__ __forceinline__ bool tail_thread(int tail) {
+  return threadIdx.y == 0 && static_cast<int>(threadIdx.x) < tail;
+}
+__device__ __forceinline__ const float* tail_column(const float4* row, int64_t cols_v) {
+  return reinterpret_cast<const float*>(row + cols_v) + threadIdx.x;
+}
+__device__ __forceinline__ float* tail_column(float4* row, int64_t cols_v) {
+  return reinterpret_cast<float*>(row + cols_v) + threadIdx.x;
+}
+
+// One column (V: of four parameters, or of one) of a group of n = 2^LOG rows: its mean.
+template <int LOG, class V>
+__device__ __forceinline__ void mean_pow2_column(V* p, int64_t ld_v) {
+  const V m = vdiv(tree_pow2<LOG>(p, ld_v), static_cast<float>(1 << LOG));
+  store_rows(p, ld_v, 1 << LOG, m);
+}
+
 // Group means, n = 2^LOG rows per group; grid.y = group index.
 template <int LOG>
 __global__ void __launch_bounds__(256) k_mean_pow2(float4* __restrict__ w, int64_t ld_v,
-                                                   int64_t cols_v) {
+                                                   int64_t cols_v, int tail) {
   grid_dep_wait();
+  float4* row = w + static_cast<int64_t>(blockIdx.y) * (int64_t(1) << LOG) * ld_v;
+  if (tail_cta(tail)) {
+    if (tail_thread(tail)) mean_pow2_column<LOG>(tail_column(row, cols_v), 4 * ld_v);
+    return;
+  }
   const int64_t c = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (c >= cols_v) return;
-  float4* p = w + static_cast<int64_t>(blockIdx.y) * (int64_t(1) << LOG) * ld_v + c;
-  const float4 m = vdiv(tree_pow2<LOG>(p, ld_v), static_cast<float>(1 << LOG));
-  store_rows(p, ld_v, 1 << LOG, m);
+  if (c < cols_v) mean_pow2_column<LOG>(row + c, ld_v);
 }
 
 // The same group sums divided by div, written once per group, to row blockIdx.y of
@@ -93,18 +119,13 @@ __global__ void __launch_bounds__(256) k_mean_pow2_to(const float4* __restrict__
 // learners each that hold the first LOGQ levels of the cluster's tree.  The result
 // is written to all P rows of w (src may be rows of w: a thread reads its column of
 // every source row before it writes).
-template <int LOGQ, int LOGS, int LOGG>
-__global__ void __launch_bounds__(256) k_local_global_pow2(const float4* src, int64_t src_ld_v,
-                                                           float4* w, int64_t ld_v, int64_t cols_v) {
-  grid_dep_wait();
-  const int64_t c = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (c >= cols_v) return;
+template <int LOGQ, int LOGS, int LOGG, class V>
+__device__ __forceinline__ void local_global_pow2_column(const V* q, int64_t src_ld_v, V* p, int64_t ld_v) {
   constexpr int S = 1 << LOGS, G = 1 << LOGG, N = 1 << (LOGS - LOGQ);
-  const float4* q = src + c;
-  float4 stack[LOGG + 1];
+  V stack[LOGG + 1];
 #pragma unroll
   for (int g = 0; g < G; ++g) {
-    float4 x = vdiv(tree_pow2<LOGS - LOGQ>(q + static_cast<int64_t>(g) * N * src_ld_v, src_ld_v),
+    V x = vdiv(tree_pow2<LOGS - LOGQ>(q + static_cast<int64_t>(g) * N * src_ld_v, src_ld_v),
                     static_cast<float>(S));
 #pragma unroll
     for (int l = 0; l < LOGS; ++l) x = vadd(x, x);
@@ -116,8 +137,23 @@ __global__ void __launch_bounds__(256) k_local_global_pow2(const float4* src, in
     }
     stack[l] = x;
   }
-  const float4 m = vdiv(stack[LOGG], static_cast<float>(S * G));
-  store_rows(w + c, ld_v, S * G, m);
+  const V m = vdiv(stack[LOGG], static_cast<float>(S * G));
+  store_rows(p, ld_v, S * G, m);
+}
+template <int LOGQ, int LOGS, int LOGG>
+__global__ void __launch_bounds__(256) k_local_global_pow2(const float4* src, int64_t src_ld_v, float4* w,
+                                                           int64_t ld_v, int64_t cols_v, int tail) {
+  grid_dep_wait();
+  if constexpr (LOGQ == 0) {             // (group sums come in whole quads)
+    if (tail_cta(tail)) {
+      if (tail_thread(tail))
+        local_global_pow2_column<LOGQ, LOGS, LOGG>(tail_column(src, cols_v), 4 * src_ld_v,
+                                                   tail_column(w, cols_v), 4 * ld_v);
+      return;
+    }
+  }
+  const int64_t c = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (c < cols_v) local_global_pow2_column<LOGQ, LOGS, LOGG>(src + c, src_ld_v, w + c, ld_v);
 }
 
 // The same two kernels with each column's rows split between two threads (threadIdx.y),
@@ -125,9 +161,15 @@ __global__ void __launch_bounds__(256) k_local_global_pow2(const float4* src, in
 // rows.  The tree over 2^LOG rows is the tree over each half joined by one addition
 // (first half + second half), so the result has the same bits.  blockDim = (128, 2).
 template <int LOG>
-__global__ void __launch_bounds__(256) k_mean_pow2_split(float4* w, int64_t ld_v, int64_t cols_v) {
+__global__ void __launch_bounds__(256) k_mean_pow2_split(float4* w, int64_t ld_v, int64_t cols_v,
+                                                         int tail) {
   __shared__ float4 part[128];
   grid_dep_wait();
+  if (tail_cta(tail)) {
+    float4* row = w + static_cast<int64_t>(blockIdx.y) * (int64_t(1) << LOG) * ld_v;
+    if (tail_thread(tail)) mean_pow2_column<LOG>(tail_column(row, cols_v), 4 * ld_v);
+    return;
+  }
   const int64_t c = static_cast<int64_t>(blockIdx.x) * 128 + threadIdx.x;
   const bool valid = c < cols_v;
   constexpr int H = 1 << (LOG - 1);
@@ -147,9 +189,17 @@ __global__ void __launch_bounds__(256) k_mean_pow2_split(float4* w, int64_t ld_v
 template <int LOGQ, int LOGS, int LOGG>
 __global__ void __launch_bounds__(256) k_local_global_pow2_split(const float4* src, int64_t src_ld_v,
                                                                  float4* w, int64_t ld_v,
-                                                                 int64_t cols_v) {
+                                                                 int64_t cols_v, int tail) {
   __shared__ float4 part[128];
   grid_dep_wait();
+  if constexpr (LOGQ == 0) {             // (group sums come in whole quads)
+    if (tail_cta(tail)) {
+      if (tail_thread(tail))
+        local_global_pow2_column<LOGQ, LOGS, LOGG>(tail_column(src, cols_v), 4 * src_ld_v,
+                                                   tail_column(w, cols_v), 4 * ld_v);
+      return;
+    }
+  }
   const int64_t c = static_cast<int64_t>(blockIdx.x) * 128 + threadIdx.x;
   const bool valid = c < cols_v;
   constexpr int S = 1 << LOGS, G2 = 1 << (LOGG - 1), N = 1 << (LOGS - LOGQ);
@@ -405,17 +455,21 @@ int ilog2_exact(int64_t n) {
 constexpr int64_t kSplitCols = 2 * 152 * 8 * 256;
 bool split_rows(int64_t cols_v, int64_t groups) { return cols_v * groups <= kSplitCols; }
 
+// Grid of the power-of-two kernels: `per` quads per CTA, and a CTA for the columns after them.
+dim3 pow2_grid(int64_t cols_v, int per, int tail, int64_t groups) {
+  return dim3(static_cast<unsigned>((cols_v + per - 1) / per + (tail != 0)), static_cast<unsigned>(groups));
+}
+
 template <int LOG>
-void launch_mean_pow2(float4* w, int64_t ld_v, int64_t cols_v, int64_t groups,
+void launch_mean_pow2(float4* w, int64_t ld_v, int64_t cols_v, int tail, int64_t groups,
                       cudaStream_t s) {
   if (split_rows(cols_v, groups)) {
-    dim3 grid(static_cast<unsigned>((cols_v + 127) / 128), static_cast<unsigned>(groups));
-    launch_pdl(k_mean_pow2_split<LOG>, grid, dim3(128, 2), 0, s, false, 1, w, ld_v, cols_v);
+    launch_pdl(k_mean_pow2_split<LOG>, pow2_grid(cols_v, 128, tail, groups), dim3(128, 2), 0, s, false, 1, w,
+               ld_v, cols_v, tail);
     return;
   }
-  dim3 grid(static_cast<unsigned>((cols_v + kThreads - 1) / kThreads),
-            static_cast<unsigned>(groups));
-  launch_pdl(k_mean_pow2<LOG>, grid, dim3(kThreads), 0, s, false, 1, w, ld_v, cols_v);
+  launch_pdl(k_mean_pow2<LOG>, pow2_grid(cols_v, kThreads, tail, groups), dim3(kThreads), 0, s, false, 1, w,
+             ld_v, cols_v, tail);
 }
 
 // (The _to launches: rows of w with stride ld_v, rows of out with stride out_ld_v.)
@@ -443,43 +497,41 @@ bool mean_pow2_to_dispatch(int log, const float4* w, int64_t ld_v, int64_t cols_
   }
 }
 
-bool mean_pow2_dispatch(int log, float4* w, int64_t ld_v, int64_t cols_v, int64_t groups,
+bool mean_pow2_dispatch(int log, float4* w, int64_t ld_v, int64_t cols_v, int tail, int64_t groups,
                         cudaStream_t s) {
   switch (log) {
-    case 1: launch_mean_pow2<1>(w, ld_v, cols_v, groups, s); return true;
-    case 2: launch_mean_pow2<2>(w, ld_v, cols_v, groups, s); return true;
-    case 3: launch_mean_pow2<3>(w, ld_v, cols_v, groups, s); return true;
-    case 4: launch_mean_pow2<4>(w, ld_v, cols_v, groups, s); return true;
-    case 5: launch_mean_pow2<5>(w, ld_v, cols_v, groups, s); return true;
-    case 6: launch_mean_pow2<6>(w, ld_v, cols_v, groups, s); return true;
-    case 7: launch_mean_pow2<7>(w, ld_v, cols_v, groups, s); return true;
+    case 1: launch_mean_pow2<1>(w, ld_v, cols_v, tail, groups, s); return true;
+    case 2: launch_mean_pow2<2>(w, ld_v, cols_v, tail, groups, s); return true;
+    case 3: launch_mean_pow2<3>(w, ld_v, cols_v, tail, groups, s); return true;
+    case 4: launch_mean_pow2<4>(w, ld_v, cols_v, tail, groups, s); return true;
+    case 5: launch_mean_pow2<5>(w, ld_v, cols_v, tail, groups, s); return true;
+    case 6: launch_mean_pow2<6>(w, ld_v, cols_v, tail, groups, s); return true;
+    case 7: launch_mean_pow2<7>(w, ld_v, cols_v, tail, groups, s); return true;
     default: return false;
   }
 }
 
 template <int LOGQ, int LOGS, int LOGG>
 void launch_lg(const float4* src, int64_t src_ld_v, float4* w, int64_t ld_v, int64_t cols_v,
-               cudaStream_t s) {
+               int tail, cudaStream_t s) {
   if constexpr (LOGG >= 1) {
     if (split_rows(cols_v, 1)) {
-      dim3 grid(static_cast<unsigned>((cols_v + 127) / 128));
-      launch_pdl(k_local_global_pow2_split<LOGQ, LOGS, LOGG>, grid, dim3(128, 2), 0, s, false, 1, src,
-                 src_ld_v, w, ld_v, cols_v);
+      launch_pdl(k_local_global_pow2_split<LOGQ, LOGS, LOGG>, pow2_grid(cols_v, 128, tail, 1), dim3(128, 2), 0,
+                 s, false, 1, src, src_ld_v, w, ld_v, cols_v, tail);
       return;
     }
   }
-  dim3 grid(static_cast<unsigned>((cols_v + kThreads - 1) / kThreads));
-  launch_pdl(k_local_global_pow2<LOGQ, LOGS, LOGG>, grid, dim3(kThreads), 0, s, false, 1, src,
-             src_ld_v, w, ld_v, cols_v);
+  launch_pdl(k_local_global_pow2<LOGQ, LOGS, LOGG>, pow2_grid(cols_v, kThreads, tail, 1), dim3(kThreads), 0, s,
+             false, 1, src, src_ld_v, w, ld_v, cols_v, tail);
 }
 
 template <int LOGQ, int LOGS>
 bool lg_dispatch_g(int logg, const float4* src, int64_t src_ld_v, float4* w, int64_t ld_v,
-                   int64_t cols_v, cudaStream_t s) {
+                   int64_t cols_v, int tail, cudaStream_t s) {
   if constexpr (LOGQ <= LOGS) {
 #define HA_LG(G_) \
     if constexpr (LOGS + G_ <= 7) \
-      if (logg == G_) { launch_lg<LOGQ, LOGS, G_>(src, src_ld_v, w, ld_v, cols_v, s); return true; }
+      if (logg == G_) { launch_lg<LOGQ, LOGS, G_>(src, src_ld_v, w, ld_v, cols_v, tail, s); return true; }
     HA_LG(0) HA_LG(1) HA_LG(2) HA_LG(3) HA_LG(4) HA_LG(5) HA_LG(6)
 #undef HA_LG
   }
@@ -488,23 +540,23 @@ bool lg_dispatch_g(int logg, const float4* src, int64_t src_ld_v, float4* w, int
 
 template <int LOGQ>
 bool lg_dispatch_s(int logs, int logg, const float4* src, int64_t src_ld_v, float4* w,
-                   int64_t ld_v, int64_t cols_v, cudaStream_t s) {
+                   int64_t ld_v, int64_t cols_v, int tail, cudaStream_t s) {
   switch (logs) {
-    case 1: return lg_dispatch_g<LOGQ, 1>(logg, src, src_ld_v, w, ld_v, cols_v, s);
-    case 2: return lg_dispatch_g<LOGQ, 2>(logg, src, src_ld_v, w, ld_v, cols_v, s);
-    case 3: return lg_dispatch_g<LOGQ, 3>(logg, src, src_ld_v, w, ld_v, cols_v, s);
-    case 4: return lg_dispatch_g<LOGQ, 4>(logg, src, src_ld_v, w, ld_v, cols_v, s);
-    case 5: return lg_dispatch_g<LOGQ, 5>(logg, src, src_ld_v, w, ld_v, cols_v, s);
+    case 1: return lg_dispatch_g<LOGQ, 1>(logg, src, src_ld_v, w, ld_v, cols_v, tail, s);
+    case 2: return lg_dispatch_g<LOGQ, 2>(logg, src, src_ld_v, w, ld_v, cols_v, tail, s);
+    case 3: return lg_dispatch_g<LOGQ, 3>(logg, src, src_ld_v, w, ld_v, cols_v, tail, s);
+    case 4: return lg_dispatch_g<LOGQ, 4>(logg, src, src_ld_v, w, ld_v, cols_v, tail, s);
+    case 5: return lg_dispatch_g<LOGQ, 5>(logg, src, src_ld_v, w, ld_v, cols_v, tail, s);
     default: return false;
   }
 }
 
 bool lg_dispatch(int logq, int logs, int logg, const float4* src, int64_t src_ld_v, float4* w,
-                 int64_t ld_v, int64_t cols_v, cudaStream_t s) {
+                 int64_t ld_v, int64_t cols_v, int tail, cudaStream_t s) {
   switch (logq) {
-    case 0: return lg_dispatch_s<0>(logs, logg, src, src_ld_v, w, ld_v, cols_v, s);
-    case 1: return lg_dispatch_s<1>(logs, logg, src, src_ld_v, w, ld_v, cols_v, s);
-    case 2: return lg_dispatch_s<2>(logs, logg, src, src_ld_v, w, ld_v, cols_v, s);
+    case 0: return lg_dispatch_s<0>(logs, logg, src, src_ld_v, w, ld_v, cols_v, tail, s);
+    case 1: return lg_dispatch_s<1>(logs, logg, src, src_ld_v, w, ld_v, cols_v, tail, s);
+    case 2: return lg_dispatch_s<2>(logs, logg, src, src_ld_v, w, ld_v, cols_v, tail, s);
     default: return false;
   }
 }
@@ -568,29 +620,17 @@ static bool vec_ok(const float* w, int64_t ld) {
   return (reinterpret_cast<uintptr_t>(w) % 16 == 0) && (ld % 4 == 0);
 }
 
-// The power-of-two kernels take aligned rows of whole quads; everything else (other group
-// sizes, other alignments) goes to the generic kernels.  A partial last quad does too, in one
-// launch, unless the matrix is so large that the power-of-two kernels' unrolled trees of 16
-// rows or more are worth a second launch for the last columns: P = 128, S = 32, D = 4000001
-// local 607 against 626 us, local + global 686 against 777; P = 64, S = 8, D = 1000001
-// local 80.7 against 76.9 us, global 114 against 103, local + global 124 against 122.
-constexpr int64_t kTailLaunch = int64_t(256) << 20;   // values in the matrix
-static bool tail_launch(int64_t rows, int64_t D) { return D % 4 != 0 && rows * D >= kTailLaunch; }
-
+// The power-of-two kernels take aligned rows; other group sizes and alignments, and rows of
+// less than a quad, go to the generic kernels.
 cudaError_t launch_group_mean(float* w, int64_t P, int64_t n, int64_t D, int64_t ld,
                               cudaStream_t s) {
   if (D == 0 || n == 1) return cudaSuccess;   // a mean of one row is that row
   const int64_t groups = P / n;
   const bool vec = vec_ok(w, ld);
   const int log = ilog2_exact(n);
-  const bool tail = n >= 16 && tail_launch(P, D);
-  int64_t head = 0;                           // columns done by a power-of-two kernel
-  if (vec && (D % 4 == 0 || tail) && log >= 1 &&
-      mean_pow2_dispatch(log, reinterpret_cast<float4*>(w), ld / 4, D / 4, groups, s))
-    head = D & ~int64_t(3);
-  if (head < D)
-    mean_any_dispatch<false>(vec, w + head, ld, D - head, static_cast<int>(n), groups,
-                             static_cast<float>(n), w + head, ld, s);
+  if (!(vec && D >= 4 && log >= 1 &&
+        mean_pow2_dispatch(log, reinterpret_cast<float4*>(w), ld / 4, D / 4, static_cast<int>(D % 4), groups, s)))
+    mean_any_dispatch<false>(vec, w, ld, D, static_cast<int>(n), groups, static_cast<float>(n), w, ld, s);
   return cudaGetLastError();
 }
 
@@ -628,14 +668,10 @@ cudaError_t launch_local_global_from_groups(const float* src, int64_t src_ld, in
   const int64_t G = P / S, n = S / Q;
   const bool vec = vec_ok(w, ld) && vec_ok(src, src_ld);
   const int logq = ilog2_exact(Q), logs = ilog2_exact(S), logg = ilog2_exact(G);
-  int64_t head = 0;
-  if (vec && (D % 4 == 0 || tail_launch(P, D)) && logq >= 0 && logs >= 1 && logg >= 0 &&
-      lg_dispatch(logq, logs, logg, reinterpret_cast<const float4*>(src), src_ld / 4,
-                  reinterpret_cast<float4*>(w), ld / 4, D / 4, s))
-    head = D & ~int64_t(3);
-  if (head < D)
-    lg_any_dispatch(vec, src + head, src_ld, static_cast<int>(n), w + head, ld, D - head,
-                    static_cast<int>(S), static_cast<int>(G), s);
+  if (!(vec && D >= 4 && (D % 4 == 0 || Q == 1) && logq >= 0 && logs >= 1 && logg >= 0 &&
+        lg_dispatch(logq, logs, logg, reinterpret_cast<const float4*>(src), src_ld / 4,
+                    reinterpret_cast<float4*>(w), ld / 4, D / 4, static_cast<int>(D % 4), s)))
+    lg_any_dispatch(vec, src, src_ld, static_cast<int>(n), w, ld, D, static_cast<int>(S), static_cast<int>(G), s);
   return cudaGetLastError();
 }
 

@@ -93,6 +93,20 @@ def test_generic_kernels(P, S, D, offset, ld_extra):
         assert np.array_equal(_bits(got), _bits(_oracle(w, op, S))), op
 
 
+# Aligned rows of odd length, group sizes that are powers of two: the columns after the last quad
+# are a CTA of their own in the same launch.  One, two and three such columns; rows of less than
+# a quad (the generic kernels) and of one; a column's rows split between two threads (up to
+# 622592 quads in all groups together) and not.
+@pytest.mark.parametrize("P,S,D,ld_extra", [
+    (4, 2, 3, 1), (8, 2, 5, 3), (8, 4, 1037, 3), (4, 4, 1022, 2), (128, 32, 515, 1), (32, 2, 131, 1),
+    (64, 16, 1025, 3), (8, 2, 622602, 2), (2, 2, 2490375, 1)])
+def test_power_of_two_groups_of_odd_rows(P, S, D, ld_extra):
+    w = replica_matrix(P, D, seed=P + D).numpy()
+    for op in ("local", "global", "local_global"):
+        got = _gpu(w, op, S, ld=D + ld_extra)
+        assert np.array_equal(_bits(got), _bits(_oracle(w, op, S))), op
+
+
 def test_edge_values():
     P, S, D = 8, 2, 64
     rng = np.random.default_rng(5)
