@@ -62,7 +62,13 @@ __device__ __forceinline__ void store_rows(V* p, int64_t ld_v, int n, V m) {
 // flight.  Rows padded to 64, this | the generic kernels | two launches: P = 16, S = 2, D =
 // 8000001 local + global 150 | 231 | 163 us; P = 64, S = 8, D = 1000003 local 74.8 | 76.8 | 80.0,
 // local + global 87.6 | 121 | 125; P = 128, S = 32, D = 4000001 local + global 618 | 777 | 689.)
-__device__ __forceinline__ bool tail_cta(int tail) { return tail != 0 && blockIdx.x == gridDim.x - 1; }
+// (kTail: kernels of their own, so that the others keep their code: D = 1000000 of 128 rows global
+// 160.4 us, 161.3 with the branch in.)
+template <bool kTail>
+__device__ __forceinline__ bool tail_cta() {
+  if constexpr (kTail) return blockIdx.x == gridDim.x - 1;
+  return false;
+}
 __device__ __forceinline__ bool tail_thread(int tail) {
   return threadIdx.y == 0 && static_cast<int>(threadIdx.x) < tail;
 }
@@ -81,12 +87,12 @@ __device__ __forceinline__ void mean_pow2_column(V* p, int64_t ld_v) {
 }
 
 // Group means, n = 2^LOG rows per group; grid.y = group index.
-template <int LOG>
+template <int LOG, bool kTail>
 __global__ void __launch_bounds__(256) k_mean_pow2(float4* __restrict__ w, int64_t ld_v,
                                                    int64_t cols_v, int tail) {
   grid_dep_wait();
   float4* row = w + static_cast<int64_t>(blockIdx.y) * (int64_t(1) << LOG) * ld_v;
-  if (tail_cta(tail)) {
+  if (tail_cta<kTail>()) {
     if (tail_thread(tail)) mean_pow2_column<LOG>(tail_column(row, cols_v), 4 * ld_v);
     return;
   }
@@ -140,17 +146,15 @@ __device__ __forceinline__ void local_global_pow2_column(const V* q, int64_t src
   const V m = vdiv(stack[LOGG], static_cast<float>(S * G));
   store_rows(p, ld_v, S * G, m);
 }
-template <int LOGQ, int LOGS, int LOGG>
+template <int LOGQ, int LOGS, int LOGG, bool kTail>
 __global__ void __launch_bounds__(256) k_local_global_pow2(const float4* src, int64_t src_ld_v, float4* w,
                                                            int64_t ld_v, int64_t cols_v, int tail) {
   grid_dep_wait();
-  if constexpr (LOGQ == 0) {             // (group sums come in whole quads)
-    if (tail_cta(tail)) {
-      if (tail_thread(tail))
-        local_global_pow2_column<LOGQ, LOGS, LOGG>(tail_column(src, cols_v), 4 * src_ld_v,
-                                                   tail_column(w, cols_v), 4 * ld_v);
-      return;
-    }
+  if (tail_cta<kTail>()) {
+    if (tail_thread(tail))
+      local_global_pow2_column<LOGQ, LOGS, LOGG>(tail_column(src, cols_v), 4 * src_ld_v, tail_column(w, cols_v),
+                                                 4 * ld_v);
+    return;
   }
   const int64_t c = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
   if (c < cols_v) local_global_pow2_column<LOGQ, LOGS, LOGG>(src + c, src_ld_v, w + c, ld_v);
@@ -160,12 +164,12 @@ __global__ void __launch_bounds__(256) k_local_global_pow2(const float4* src, in
 // for short rows (D small against the GPU): twice the threads, each walking half the
 // rows.  The tree over 2^LOG rows is the tree over each half joined by one addition
 // (first half + second half), so the result has the same bits.  blockDim = (128, 2).
-template <int LOG>
+template <int LOG, bool kTail>
 __global__ void __launch_bounds__(256) k_mean_pow2_split(float4* w, int64_t ld_v, int64_t cols_v,
                                                          int tail) {
   __shared__ float4 part[128];
   grid_dep_wait();
-  if (tail_cta(tail)) {
+  if (tail_cta<kTail>()) {
     float4* row = w + static_cast<int64_t>(blockIdx.y) * (int64_t(1) << LOG) * ld_v;
     if (tail_thread(tail)) mean_pow2_column<LOG>(tail_column(row, cols_v), 4 * ld_v);
     return;
@@ -186,19 +190,17 @@ __global__ void __launch_bounds__(256) k_mean_pow2_split(float4* w, int64_t ld_v
 
 // (threadIdx.y = which half of the G clusters; the first G / 2 clusters' S copies form a
 // complete sub-tree of the global tree.)
-template <int LOGQ, int LOGS, int LOGG>
+template <int LOGQ, int LOGS, int LOGG, bool kTail>
 __global__ void __launch_bounds__(256) k_local_global_pow2_split(const float4* src, int64_t src_ld_v,
                                                                  float4* w, int64_t ld_v,
                                                                  int64_t cols_v, int tail) {
   __shared__ float4 part[128];
   grid_dep_wait();
-  if constexpr (LOGQ == 0) {             // (group sums come in whole quads)
-    if (tail_cta(tail)) {
-      if (tail_thread(tail))
-        local_global_pow2_column<LOGQ, LOGS, LOGG>(tail_column(src, cols_v), 4 * src_ld_v,
-                                                   tail_column(w, cols_v), 4 * ld_v);
-      return;
-    }
+  if (tail_cta<kTail>()) {
+    if (tail_thread(tail))
+      local_global_pow2_column<LOGQ, LOGS, LOGG>(tail_column(src, cols_v), 4 * src_ld_v, tail_column(w, cols_v),
+                                                 4 * ld_v);
+    return;
   }
   const int64_t c = static_cast<int64_t>(blockIdx.x) * 128 + threadIdx.x;
   const bool valid = c < cols_v;
@@ -464,12 +466,12 @@ template <int LOG>
 void launch_mean_pow2(float4* w, int64_t ld_v, int64_t cols_v, int tail, int64_t groups,
                       cudaStream_t s) {
   if (split_rows(cols_v, groups)) {
-    launch_pdl(k_mean_pow2_split<LOG>, pow2_grid(cols_v, 128, tail, groups), dim3(128, 2), 0, s, false, 1, w,
-               ld_v, cols_v, tail);
+    launch_pdl(tail != 0 ? k_mean_pow2_split<LOG, true> : k_mean_pow2_split<LOG, false>,
+               pow2_grid(cols_v, 128, tail, groups), dim3(128, 2), 0, s, false, 1, w, ld_v, cols_v, tail);
     return;
   }
-  launch_pdl(k_mean_pow2<LOG>, pow2_grid(cols_v, kThreads, tail, groups), dim3(kThreads), 0, s, false, 1, w,
-             ld_v, cols_v, tail);
+  launch_pdl(tail != 0 ? k_mean_pow2<LOG, true> : k_mean_pow2<LOG, false>,
+             pow2_grid(cols_v, kThreads, tail, groups), dim3(kThreads), 0, s, false, 1, w, ld_v, cols_v, tail);
 }
 
 // (The _to launches: rows of w with stride ld_v, rows of out with stride out_ld_v.)
@@ -514,15 +516,17 @@ bool mean_pow2_dispatch(int log, float4* w, int64_t ld_v, int64_t cols_v, int ta
 template <int LOGQ, int LOGS, int LOGG>
 void launch_lg(const float4* src, int64_t src_ld_v, float4* w, int64_t ld_v, int64_t cols_v,
                int tail, cudaStream_t s) {
+  constexpr bool kTail = LOGQ == 0;      // (group sums come in whole quads)
   if constexpr (LOGG >= 1) {
     if (split_rows(cols_v, 1)) {
-      launch_pdl(k_local_global_pow2_split<LOGQ, LOGS, LOGG>, pow2_grid(cols_v, 128, tail, 1), dim3(128, 2), 0,
-                 s, false, 1, src, src_ld_v, w, ld_v, cols_v, tail);
+      launch_pdl(tail != 0 ? k_local_global_pow2_split<LOGQ, LOGS, LOGG, kTail>
+                           : k_local_global_pow2_split<LOGQ, LOGS, LOGG, false>,
+                 pow2_grid(cols_v, 128, tail, 1), dim3(128, 2), 0, s, false, 1, src, src_ld_v, w, ld_v, cols_v, tail);
       return;
     }
   }
-  launch_pdl(k_local_global_pow2<LOGQ, LOGS, LOGG>, pow2_grid(cols_v, kThreads, tail, 1), dim3(kThreads), 0, s,
-             false, 1, src, src_ld_v, w, ld_v, cols_v, tail);
+  launch_pdl(tail != 0 ? k_local_global_pow2<LOGQ, LOGS, LOGG, kTail> : k_local_global_pow2<LOGQ, LOGS, LOGG, false>,
+             pow2_grid(cols_v, kThreads, tail, 1), dim3(kThreads), 0, s, false, 1, src, src_ld_v, w, ld_v, cols_v, tail);
 }
 
 template <int LOGQ, int LOGS>
