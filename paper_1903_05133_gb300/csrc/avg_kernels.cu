@@ -238,13 +238,13 @@ __global__ void __launch_bounds__(256) k_local_global_pow2_split(const float4* s
 // columns, which an access policy maps to memory: Quad for rows that start on 16 bytes (four
 // neighbours, one 128-bit access; the row's last quad may be partial), Spread for all others
 // (columns 256 apart, so that each of the four 32-bit accesses of a warp is contiguous).
-// Everything lives in registers: the tree over n rows is the tree over the complete block of
-// each set bit of n, highest bit first, folded from the smallest block upward (the binary
-// counter's pending partials), and each block is unrolled with its loads in flight.  (One
-// column per thread with the counter in a local array had been bound by the latency of its
-// serial loads and stack.  Unaligned rows, L2 holding the matrix: P = 12, S = 6, D = 1000003
-// local 23.4 -> 12.5 us, local + global 34.0 -> 17.0 us (5.6 TB/s); P = 48, S = 8, D = 8000001
-// from HBM: local 905 -> 459 us (6.7 TB/s), global 880 -> 622, local + global 1067 -> 699.)
+// The tree over n rows is the tree over the complete block of each set bit of n, highest bit
+// first, folded from the smallest block upward (the binary counter's pending partials), and each
+// block is unrolled in registers with its loads in flight.  (One column per thread with the
+// counter in a local array had been bound by the latency of its serial loads and stack.
+// Unaligned rows, L2 holding the matrix: P = 12, S = 6, D = 1000003 local 23.4 -> 12.5 us, local +
+// global 34.0 -> 17.0 us (5.6 TB/s); P = 48, S = 8, D = 8000001 from HBM: local 905 -> 459 us
+// (6.7 TB/s), global 880 -> 622, local + global 1067 -> 699.)
 struct Quad {
   using V = float4;
   static constexpr int kCols = 4;
@@ -325,21 +325,29 @@ __device__ __forceinline__ typename A::V tree_block(const A& a, const float* p, 
 
 // The binary counter over values pushed in order, with blocks of 2^level values that are
 // equal or already summed pushed at once (idx: the block's first value, a multiple of
-// 2^level).  The levels are unrolled and uniform over the CTA, so the partials stay in
-// registers.
-template <class V, int LEVELS>
+// 2^level).  The levels are uniform over the CTA.  Unrolled, the partials stay in registers and a
+// push costs every level's test; kLoop, a push ends at the level where its block comes to rest
+// (every other one at its first) and the partials stand in local memory, where a thread's few
+// live ones stay in L1: better for many pushes of small blocks.
+template <class V, int LEVELS, bool kLoop = false>
 struct Counter {
   V st[LEVELS];
   __device__ __forceinline__ void push(int idx, int level, V x) {
-    bool open = true;
+    if constexpr (kLoop) {
+      int l = level;
+      for (; (idx >> l) & 1; ++l) x = vadd(st[l], x);
+      st[l] = x;
+    } else {
+      bool open = true;
 #pragma unroll
-    for (int l = 0; l < LEVELS; ++l) {
-      if (l < level || !open) continue;
-      if ((idx >> l) & 1) {
-        x = vadd(st[l], x);
-      } else {
-        st[l] = x;
-        open = false;
+      for (int l = 0; l < LEVELS; ++l) {
+        if (l < level || !open) continue;
+        if ((idx >> l) & 1) {
+          x = vadd(st[l], x);
+        } else {
+          st[l] = x;
+          open = false;
+        }
       }
     }
   }
@@ -413,17 +421,20 @@ __global__ void __launch_bounds__(256) k_mean_any(const float* src, int64_t ld, 
 // (src, src_ld, n: as in k_local_global_pow2, n = S / Q source rows per cluster.)  The global
 // tree runs over S copies of each cluster mean; a complete block of 2^l copies is the mean
 // added to itself l times, so a cluster's run is pushed as its maximal aligned blocks.
-// (BITS: of n; LEVELS: of P.  Three CTAs per SM: without the limit the compiler keeps so many
-// rows in flight per thread that one fits, and P = 24, S = 4, D = 5025045 took 407 instead of
-// 190 us.)
+// (BITS: of n; LEVELS: of P.  Up to 255 rows, three CTAs per SM: without the limit the compiler
+// keeps so many rows in flight per thread that one fits, and P = 24, S = 4, D = 5025045 took 407
+// instead of 190 us; the kernels for clusters of 16 rows and more spill under it.  Clusters of
+// less than 16 rows are many pushes, a looped counter's: P = 48, S = 3, D = 1000003 with padded
+// rows 120 -> 67 us.  From 16 rows on there are few, and unrolled levels are as fast or faster up
+// to 8 of them (P = 96, S = 96, D = 262145 42.0 us against 47.5 looped), looped ones beyond.)
 template <class A, int BITS, int LEVELS>
-__global__ void __launch_bounds__(256, LEVELS == 4 ? 4 : LEVELS == 8 ? 3 : 1) k_local_global_any(const float* src, int64_t src_ld, int n,
-                                                          float* w, int64_t ld, int64_t cols, int S,
-                                                          int G) {
+__global__ void __launch_bounds__(256, LEVELS == 4 ? 4 : LEVELS == 8 ? 3 : 1)
+    k_local_global_any(const float* src, int64_t src_ld, int n, float* w, int64_t ld, int64_t cols, int S,
+                       int G) {
   grid_dep_wait();
   const A a(cols);
   if (a.live == 0) return;
-  Counter<typename A::V, LEVELS> cnt;
+  Counter<typename A::V, LEVELS, (LEVELS > (BITS == 4 ? 4 : 8))> cnt;
   for (int g = 0; g < G; ++g) {
     const typename A::V m =
         vdiv(tree_rows<BITS, false>(a, src + static_cast<int64_t>(g) * n * src_ld, src_ld, n),
@@ -604,17 +615,31 @@ void launch_lg_any(const float* src, int64_t src_ld, int n, float* w, int64_t ld
              any_grid<A>(cols, 1), dim3(256), 0, s, false, 1, src, src_ld, n, w, ld, cols, S, G);
 }
 
+// From 256 rows on, four columns per thread only where clusters of less than 16 rows leave the
+// registers for it and the row gives every SM two CTAs: local + global, D = 1000000, quads | one
+// column per thread: P = 256, S = 16 749 | 370 us; P = 512, S = 64 1361 | 696.  (Before, | one
+// kernel with 31 unrolled levels for all of them, | a counter in a local array for all sizes:
+// P = 512, S = 2, D = 1000001 735 | 5310 | 1508 us, P = 300, S = 3, D = 1000000 436 | 3554 | 699,
+// P = 300, S = 75 440 | 746 | 614, P = 5000, S = 2, D = 65600 1988 | 4169 | 4456.)
 void lg_any_dispatch(bool vec, const float* src, int64_t src_ld, int n, float* w, int64_t ld,
                      int64_t cols, int S, int G, cudaStream_t s) {
-  if (static_cast<int64_t>(S) * G >= 256)
-    launch_pdl(k_local_global_any<Single, 31, 31>, any_grid<Single>(cols, 1), dim3(256), 0, s, false, 1, src,
-               src_ld, n, w, ld, cols, S, G);
-  else if (vec)
-    launch_lg_any<Quad>(src, src_ld, n, w, ld, cols, S, G, s);
-  else if (spread_wide(cols, 1))
-    launch_lg_any<Spread>(src, src_ld, n, w, ld, cols, S, G, s);
-  else
-    launch_lg_any<Single>(src, src_ld, n, w, ld, cols, S, G, s);
+  const int64_t P = static_cast<int64_t>(S) * G;
+  const bool wide = spread_wide(cols, 1);
+  if (P < 256) {
+    if (vec)
+      launch_lg_any<Quad>(src, src_ld, n, w, ld, cols, S, G, s);
+    else if (wide)
+      launch_lg_any<Spread>(src, src_ld, n, w, ld, cols, S, G, s);
+    else
+      launch_lg_any<Single>(src, src_ld, n, w, ld, cols, S, G, s);
+  } else if (P < 4096 && n < 16 && wide) {
+    launch_pdl(vec ? k_local_global_any<Quad, 4, 12> : k_local_global_any<Spread, 4, 12>, any_grid<Quad>(cols, 1),
+               dim3(256), 0, s, false, 1, src, src_ld, n, w, ld, cols, S, G);
+  } else {
+    launch_pdl(P < 4096 ? n < 16 ? k_local_global_any<Single, 4, 12> : k_local_global_any<Single, 12, 12>
+                        : n < 16 ? k_local_global_any<Single, 4, 31> : k_local_global_any<Single, 31, 31>,
+               any_grid<Single>(cols, 1), dim3(256), 0, s, false, 1, src, src_ld, n, w, ld, cols, S, G);
+  }
 }
 
 }  // namespace

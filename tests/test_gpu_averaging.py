@@ -93,6 +93,22 @@ def test_generic_kernels(P, S, D, offset, ld_extra):
         assert np.array_equal(_bits(got), _bits(_oracle(w, op, S))), op
 
 
+# The fused average over many clusters: small ones (a looped counter) and clusters of 16 rows
+# and more, under and from 256 and 4096 rows on, the last columns of rows on both sides of the
+# four-columns-per-thread limit, aligned and not.  The oracle checks a sample of the columns.
+@pytest.mark.parametrize("P,S,D,ld", [
+    (24, 3, 40001, 40001), (250, 2, 1003, 1024), (48, 3, 311299, 311300), (255, 17, 1001, 1001),
+    (256, 2, 311300, 311300), (300, 3, 311299, 311299), (258, 43, 311299, 311299), (512, 16, 515, 516),
+    (1023, 3, 130, 131), (4095, 5, 33, 36), (4096, 2, 130, 130), (5000, 2500, 67, 67)])
+def test_local_global_of_many_clusters(P, S, D, ld):
+    torch.manual_seed(P + D)
+    w = torch.randn(P, ld, device="cuda")[:, :D]
+    cols = torch.cat([torch.randint(0, D, (64,), device="cuda"), torch.arange(D - 8, D, device="cuda")])
+    src = w[:, cols].cpu().numpy()
+    ha.local_global_average_buffer(w, S)
+    assert np.array_equal(_bits(w[:, cols].cpu().numpy()), _bits(_oracle(src, "local_global", S)))
+
+
 # Aligned rows of odd length, group sizes that are powers of two: the columns after the last quad
 # are a CTA of their own in the same launch.  One, two and three such columns; rows of less than
 # a quad (the generic kernels) and of one; a column's rows split between two threads (up to
