@@ -276,15 +276,18 @@ void plan_layout(hier_avg* h, bool fine = true) {
         // Few long tiles (at most kPieceChunks chunks, so whole tiles otherwise) in pieces of
         // one promotion segment, kFineChunks chunks, while every piece has an SM of its own.
         // The partials are the segment sums that a whole tile adds in the same order, so dX
-        // keeps its bits.  The partials' round trip costs about 12 chunks' time (B <= 32; more
-        // for larger batches): P = 2, a round of 6 steps of 784-512-n-10, B = 32: n = 512
+        // keeps its bits.  The partials' round trip costs about 12 chunks' time at B <= 32 and
+        // grows with the batch.  P = 2, a round of 6 steps of 784-512-n-10, B = 32: n = 512
         // (8 chunks) 456 -> 464 us, 1000 (16) 416 -> 419, 1200 (19) 570 -> 517, 1536 (24) 545 ->
-        // 432, 2504 (40) 603 -> 500; B = 64: 1200 703 -> 723, 1536 680 -> 625.  Pieces in two
-        // turns lost as often as they won (P = 4, B = 48, 2512: 786 -> 803; P = 8, B = 32, 2048:
-        // 630 -> 528).
+        // 432, 2504 (40) 603 -> 500.  4 steps, P = 1, 2, 3, 4: B = 48, 1536 304 -> 309 (P = 3), 432
+        // -> 417 (4), 2048 399 -> 385, 336 -> 325, 371 -> 365, 449 -> 388; B = 64, 1536 348 -> 367,
+        // 396 -> 417, 337 -> 392, 484 -> 466, 2048 450 -> 457, 367 -> 378, 407 -> 425, 487 -> 447,
+        // 2504 560 -> 537, 483 -> 472, 486 -> 467.  Pieces in two turns lost as often as they won
+        // (P = 4, B = 48, 2512: 786 -> 803; P = 8, B = 32, 2048: 630 -> 528).
         int64_t pc = kPieceChunks;
         const int64_t fp = (nc + kFineChunks - 1) / kFineChunks;
-        if (fine && l > 0 && nc <= kPieceChunks && nc >= (h->Bn <= 32 ? 17 : 24) && btiles * P * fp <= kTargetCtas) {
+        const int64_t nc_min = h->Bn <= 32 ? 17 : h->Bn <= 48 ? 24 : 32;
+        if (fine && l > 0 && nc >= nc_min && nc <= kPieceChunks && btiles * P * fp <= kTargetCtas) {
           pc = kFineChunks;
           fine_used = true;
         }

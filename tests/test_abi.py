@@ -74,6 +74,30 @@ def test_layout_and_workspace(lib):
         lib.hier_avg_destroy(h)
 
 
+# Where the backward of few long tiles goes in pieces, the workspace holds the pieces' partials
+# (P tiles of 256 inputs in ceil(chunks / 4) pieces of 128 x Bn floats): from 17 chunks of 64
+# outputs on up to 32 samples, from 24 up to 48, from 32 up to 64.
+@pytest.mark.parametrize("B,first", [(16, 17), (32, 17), (48, 24), (64, 32)])
+def test_partials_of_backward_pieces_are_reserved_from(lib, B, first):
+    P = 2
+
+    def step_bytes(chunks):
+        rc, h = _create(lib, P=P, S=1, B=B, dims=(64, 256, 64 * chunks, 10))
+        assert rc == 0
+        wb = ctypes.c_int64()
+        assert lib.hier_avg_workspace_bytes(h, ctypes.byref(wb)) == 0
+        lib.hier_avg_destroy(h)
+        return wb.value - 2 * P * B * 64 * chunks * 2            # without H_2 and dZ_2
+
+    def partials(chunks):
+        return 2 * P * ((chunks + 3) // 4) * 128 * B * 4
+
+    slack = 4096                                                 # counters, alignment
+    assert abs(step_bytes(first - 1) - step_bytes(first - 2)) <= slack
+    assert abs(step_bytes(first) - step_bytes(first - 1) - partials(first)) <= slack
+    assert abs(step_bytes(48) - step_bytes(first) - partials(48) + partials(first)) <= slack
+
+
 def test_calls_before_bind_fail_cleanly(lib):
     rc, h = _create(lib)
     assert rc == 0
