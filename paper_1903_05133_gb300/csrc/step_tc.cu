@@ -17,6 +17,7 @@
 //             dW^T = H^T dZ, the fp32 update of W, and dH^T += W_q^T dZ^T;
 //             epilogue dZ_{l-1} = dH [H_{l-1} > 0], b_{l-1} -= lr sum_b dZ_{l-1}.
 // W is read once by the forward and once (read, written) by the backward.
+#include <algorithm>
 #include <cstdint>
 #include <cuda.h>
 #include <cuda_bf16.h>
@@ -2701,11 +2702,10 @@ __global__ void __launch_bounds__(kXentThreads, 1) k_xent_bf16(const float* __re
 // b_L -= lr * sum_b dZ (in sample order).  Rank 0 also writes the learner's mean loss.  Bound by
 // the exponentials, divisions and dependent loads of a sample, which one CTA keeps on one SM
 // (P = 32, 1000 classes, B = 32: 22.9 -> 12.9 us per launch; P = 2, 400 classes, B = 64: 3 steps
-// 286 -> 265 us).  Below about 12 K logits per learner the cluster's launch and barrier cost what
-// it saves or more (P = 32, 300 classes, B = 16: 7.7 against 7.2 us per launch; P = 2, 622
-// classes, B = 16: 7.9 against 8.2; P = 64, 348, B = 16: a round of 18 steps 356.3 against 358.8).
+// 286 -> 265 us).  xent_spread says where it is the faster one.
 constexpr int kXentcThreads = 256, kXentRanks = 8, kXentTile = 128;
 constexpr int kXentSpread = 12288;               // logits per learner
+constexpr int kXentSms = 152;                    // of a GB300
 __global__ void __launch_bounds__(kXentcThreads) k_xent_bf16_cluster(const float* __restrict__ Z,
                                                            const int32_t* __restrict__ y,
                                                            int64_t N, int64_t row0, int B, int Bn,
@@ -2935,11 +2935,30 @@ cudaError_t launch_gather_bf16(const __nv_bfloat16* X, int64_t N, int d0, int B,
   return launch_pdl(k_gather_bf16, grid, dim3(256), 0, s, false, 1, X, N, d0, B, Bn, pitch0, row0, H0);
 }
 
+// Whether the cross-entropy of a learner goes over a cluster.  Below about 12 K logits the
+// cluster's launch and barrier cost what it saves or more (us per launch, cluster | one CTA per
+// 1024 classes: P = 32, 300 classes, B = 16 7.7 | 7.2; P = 2, 622 classes 7.9 | 8.2).  While the
+// other kernel's CTAs take one wave, they have 32 warps each for the samples' statistics against
+// the ranks' 8, and 1024 classes each: few samples or many classes are theirs (P = 16: B = 32, 1000
+// classes 15.5 | 18.5, 2000 24.4 | 22.5; B = 64, 3000 45.8 | 47.1, 4000 57.8 | 55.3; B = 16, 2000
+// 19.1 | 16.3), and many learners, whose clusters are several CTAs per SM (B = 32, 1000 classes:
+// P = 48 16.5 | 18.5, 64 18.3 | 18.4, 96 22.3 | 18.4, 128 28.7 | 18.4).  In two waves and more of
+// them the cluster wins, unless there are so many learners that its own CTAs are five or more to
+// an SM (B = 16: P = 64, 3000 classes 28.8 | 32.8; P = 128, 2000 35.5 | 28.7, 4000 63.6 | 77.9; P =
+// 160, 1000 24.3 | 22.0; B = 48: P = 128, 2000 63.1 | 62.5, P = 160, 1000 38.8 | 45.1; P = 256, 1000
+// 56.7 | 47.1, 2000 104 | 132).
+static bool xent_spread(int64_t P, int64_t B, int64_t C) {
+  if (B * C < kXentSpread) return false;
+  const int64_t waves = (P * ((C + kXentThreads - 1) / kXentThreads) + kXentSms - 1) / kXentSms;
+  if (waves == 1) return P <= 64 && C * std::max<int64_t>(P, 32) <= 1536 * B;
+  return kXentSms * waves >= 3 * P || (B >= 48 && 5 * kXentSms * waves >= 9 * P);
+}
+
 cudaError_t launch_xent_bf16(const float* Z, const int32_t* y, int64_t N, int64_t row0, int B,
                              int Bn, int C, int pitch_c, float lr, const float* bias_src,
                              int src_div, float* bias_L, int64_t ld, __nv_bfloat16* dZ,
                              float* loss, int P, cudaStream_t s) {
-  if (static_cast<int64_t>(B) * C >= kXentSpread)
+  if (xent_spread(P, B, C))
     return launch_pdl(k_xent_bf16_cluster, dim3(kXentRanks, P), dim3(kXentcThreads), 0, s, false, kXentRanks, Z, y,
                       N, row0, B, Bn, C, pitch_c, lr, bias_src, src_div, bias_L, ld, dZ, loss);
   dim3 grid(P, (C + kXentThreads - 1) / kXentThreads);

@@ -792,13 +792,17 @@ def test_backward_in_segment_pieces(w):
 # The cross-entropy over a cluster: fewer samples than its CTAs, a last CTA with fewer than
 # the others, more samples than threads, just past and just below the logits from which on it is
 # spread (12288), class slices of one partial tile and of more than one tile of 128 with an odd rest.
+# In bf16 with one wave of the other kernel's CTAs up to 48 classes per sample, both sides of that;
+# few samples where those CTAs are more than a wave.
 # (300 samples: the mean gradient is small, and the update's bound of 1e-5 has to hold over half
 # an ulp of a weight of 0.6, 3e-8: at lr = 0.05 that is 1.2e-5 of the update, at 1 6e-7.)
 XENT_CASES = [_fp32((40, 36, 1500), 2, 1, 9), _fp32((64, 65), 2, 1, 300).replace(lr=1.0),
               _fp32((40, 33), 3, 1, 373).replace(lr=1.0), _fp32((40, 33), 3, 1, 372).replace(lr=1.0),
               _small((64, 72, 2459), "bf16", 2, 2, 5, 2, 20), _small((64, 72, 1100), "bf16", 3, 1, 64, 2, 130),
               _small((72, 2056), "bf16", 2, 1, 33, 1, 50), _small((64, 136, 193), "bf16", 2, 2, 64, 2, 130),
-              _small((64, 136, 191), "bf16", 2, 2, 64, 2, 130)]
+              _small((64, 136, 191), "bf16", 2, 2, 64, 2, 130), _small((64, 64, 3073), "bf16", 64, 8, 4, 2, 16),
+              _small((64, 64, 1025), "bf16", 100, 4, 13, 2, 40), _small((64, 72, 1537), "bf16", 2, 2, 32, 2, 70),
+              _small((64, 72, 1536), "bf16", 2, 2, 32, 2, 70)]
 
 
 @pytest.mark.parametrize("w", XENT_CASES, ids=lambda w: w.name)
