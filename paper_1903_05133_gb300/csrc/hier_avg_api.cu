@@ -14,6 +14,7 @@
 #include <cuda.h>
 #include <cuda_runtime.h>
 
+#include "context_once.h"
 #include "internal.h"
 #include "ptx.cuh"
 
@@ -45,6 +46,34 @@ EncodeTiledFn encode_fn() {
       fn = reinterpret_cast<EncodeTiledFn>(p);
   }
   return fn;
+}
+
+typedef CUresult (*CtxGetCurrentFn)(CUcontext*);
+typedef CUresult (*CtxGetIdFn)(CUcontext, unsigned long long*);
+
+// Unique id of the current CUDA context (ids are never reused within a process), or
+// 0 if it cannot be read.
+unsigned long long current_context_id() {
+  static CtxGetCurrentFn get_current = nullptr;
+  static CtxGetIdFn get_id = nullptr;
+  static std::once_flag once;
+  std::call_once(once, [] {
+    cudaDriverEntryPointQueryResult q;
+    void* p = nullptr;
+    if (cudaGetDriverEntryPointByVersion("cuCtxGetCurrent", &p, 12000, cudaEnableDefault, &q) ==
+            cudaSuccess && q == cudaDriverEntryPointSuccess)
+      get_current = reinterpret_cast<CtxGetCurrentFn>(p);
+    p = nullptr;
+    if (cudaGetDriverEntryPointByVersion("cuCtxGetId", &p, 12000, cudaEnableDefault, &q) ==
+            cudaSuccess && q == cudaDriverEntryPointSuccess)
+      get_id = reinterpret_cast<CtxGetIdFn>(p);
+  });
+  CUcontext ctx = nullptr;
+  unsigned long long id = 0;
+  if (!get_current || !get_id || get_current(&ctx) != CUDA_SUCCESS || !ctx ||
+      get_id(ctx, &id) != CUDA_SUCCESS)
+    return 0;
+  return id;
 }
 
 struct ProfRec {
@@ -417,15 +446,25 @@ int build_maps(hier_avg* h) {
   return HA_OK;
 }
 
-// Attributes of the kernels that the handle's steps launch, and their tensor maps (small nets
-// use none).
+ha::ContextOnce g_attributes;
+
+// Attributes of the kernels that the handle's steps launch, set once per context: eleven calls
+// for the fp32 path, 3.5 us of every bind and every static step before.
+int kernel_attributes(hier_avg* h) {
+  const bool bf16 = h->prec == HA_PREC_BF16;
+  const int e = g_attributes.run(current_context_id(), h->small ? 1 : bf16 ? 2 : 4, [&]() -> int {
+    if (h->small) return ha::small_configure();
+    if (!bf16) return ha::fp32_configure();
+    const cudaError_t rc = ha::tc_configure();
+    return rc != cudaSuccess ? rc : ha::head_configure();
+  });
+  return h->cuda(static_cast<cudaError_t>(e), "kernel attributes");
+}
+
+// Kernel attributes and tensor maps (small nets and the fp32 path use none).
 int configure(hier_avg* h) {
-  const char* what = "kernel attributes";
-  if (h->small) return h->cuda(ha::small_configure(), what);
-  if (h->prec != HA_PREC_BF16) return h->cuda(ha::fp32_configure(), what);
-  if (int rc = h->cuda(ha::tc_configure(), what)) return rc;
-  if (int rc = h->cuda(ha::head_configure(), what)) return rc;
-  return build_maps(h);
+  if (int rc = kernel_attributes(h)) return rc;
+  return h->small || h->prec != HA_PREC_BF16 ? HA_OK : build_maps(h);
 }
 
 int check_bound(hier_avg* h) {
@@ -1498,34 +1537,6 @@ int hier_avg_profile_read(hier_avg* h, int kind, double* total_ms, int64_t* laun
 namespace {
 
 static __device__ __align__(256) unsigned char g_static_scratch[kStaticScratchBytes];
-
-typedef CUresult (*CtxGetCurrentFn)(CUcontext*);
-typedef CUresult (*CtxGetIdFn)(CUcontext, unsigned long long*);
-
-// Unique id of the current CUDA context (ids are never reused within a process), or
-// 0 if it cannot be read.
-unsigned long long current_context_id() {
-  static CtxGetCurrentFn get_current = nullptr;
-  static CtxGetIdFn get_id = nullptr;
-  static std::once_flag once;
-  std::call_once(once, [] {
-    cudaDriverEntryPointQueryResult q;
-    void* p = nullptr;
-    if (cudaGetDriverEntryPointByVersion("cuCtxGetCurrent", &p, 12000, cudaEnableDefault, &q) ==
-            cudaSuccess && q == cudaDriverEntryPointSuccess)
-      get_current = reinterpret_cast<CtxGetCurrentFn>(p);
-    p = nullptr;
-    if (cudaGetDriverEntryPointByVersion("cuCtxGetId", &p, 12000, cudaEnableDefault, &q) ==
-            cudaSuccess && q == cudaDriverEntryPointSuccess)
-      get_id = reinterpret_cast<CtxGetIdFn>(p);
-  });
-  CUcontext ctx = nullptr;
-  unsigned long long id = 0;
-  if (!get_current || !get_id || get_current(&ctx) != CUDA_SUCCESS || !ctx ||
-      get_id(ctx, &id) != CUDA_SUCCESS)
-    return 0;
-  return id;
-}
 
 std::mutex g_scratch_mutex;
 struct ScratchAddr {
