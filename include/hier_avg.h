@@ -100,7 +100,8 @@ int hier_avg_param_layout(const hier_avg* h, int64_t* D, int64_t* ld, int64_t* o
 
 /* Bytes of device workspace hier_avg_bind needs: a step's scratch and, for the bf16
  * path with S > 1, the cluster means [P / S, ld] fp32 that hier_avg_round's local
- * averages write. */
+ * averages write.  (Small nets, whose steps keep everything else in shared memory, need
+ * the losses and the error word only, and average in place.) */
 int hier_avg_workspace_bytes(const hier_avg* h, int64_t* bytes);
 
 /* Attach device memory (all borrowed, caller-owned) and the stream:

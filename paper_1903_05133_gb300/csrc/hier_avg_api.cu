@@ -237,7 +237,22 @@ void plan_layout(hier_avg* h, bool fine = true) {
   h->off_H.assign(L + 1, 0);
   h->off_dZ.assign(L + 1, 0);
   h->pitch.assign(L + 1, 0);
-  if (h->prec == HA_PREC_BF16) {
+  const bool bf16 = h->prec == HA_PREC_BF16;
+  const int wl = h->dims[L - 1];
+  // Last layers of up to 16 classes run as one kernel.  In bf16, where the width is no multiple
+  // of 64, that replaces the tensor-core forward and backward with their partly filled tiles:
+  // 264-136-200-13 (P = 6, B = 20) 55 -> 43 us per step, one-layer 784-10 (P = 24, B = 64)
+  // 43 -> 15 us.  Wide layers after hidden ones keep the tensor-core kernels, whose tiles
+  // are nearly full there (2512 -> 10 behind 3072-512, P = 4: 1.6 % of the step).
+  h->head = bf16 ? (wl % 64 == 0 || L == 1 || wl <= 1024) &&
+                       ha::head_supported(h->dims[L], wl, static_cast<int>(B), h->P)
+                 : ha::head32_supported(h->dims[L], wl, static_cast<int>(B));
+  h->small = !(h->head && L == 1) &&
+             ha::small_supported(h->dims.data(), L, static_cast<int>(B), h->P, bf16);
+  if (h->small) {
+    // (the one kernel keeps activations, gradients and partials in shared memory, and its
+    // averages write every row)
+  } else if (bf16) {
     h->Bn = static_cast<int>(round_up(B, 16));
     for (int l = 0; l <= L; ++l) h->pitch[l] = static_cast<int>(round_up(h->dims[l], 64));
     for (int l = 0; l < L; ++l) h->off_H[l] = take(P * h->Bn * h->pitch[l] * 2);
@@ -332,32 +347,21 @@ void plan_layout(hier_avg* h, bool fine = true) {
       max_tiles = std::max(max_tiles, std::max(ftiles, btiles) * P);
     }
     h->fused_xent = h->dims[L] <= 128;
-    // Last layers of up to 16 classes run as one kernel.  Where the width is no multiple of
-    // 64 that replaces the tensor-core forward and backward with their partly filled tiles:
-    // 264-136-200-13 (P = 6, B = 20) 55 -> 43 us per step, one-layer 784-10 (P = 24, B = 64)
-    // 43 -> 15 us.  Wide layers after hidden ones keep the tensor-core kernels, whose tiles
-    // are nearly full there (2512 -> 10 behind 3072-512, P = 4: 1.6 % of the step).
-    const int64_t wl = h->dims[L - 1];
-    h->head = (wl % 64 == 0 || L == 1 || wl <= 1024) &&
-              ha::head_supported(h->dims[L], h->dims[L - 1], static_cast<int>(B), h->P);
     h->off_part = take(part_bytes);
     h->off_cnt = take(max_tiles * 4);
     h->off_dyn = take(16);
   } else {
-    for (int l = 0; l <= L; ++l) h->pitch[l] = h->dims[l];
-    h->head = ha::head32_supported(h->dims[L], h->dims[L - 1], static_cast<int>(B));
-    for (int l = 0; l < L; ++l) h->off_H[l] = take(P * B * h->dims[l] * 4);
-    for (int l = 1; l <= L; ++l) h->off_dZ[l] = take(P * B * h->dims[l] * 4);
+    // (the first layer reads X itself, and the last layer's kernel writes neither Z nor dZ_L)
+    for (int l = 1; l < L; ++l) h->off_H[l] = take(P * B * h->dims[l] * 4);
+    for (int l = 1; l < L + !h->head; ++l) h->off_dZ[l] = take(P * B * h->dims[l] * 4);
   }
-  h->small = !(h->head && L == 1) &&
-             ha::small_supported(h->dims.data(), L, static_cast<int>(B), h->P, h->prec == HA_PREC_BF16);
-  h->off_Z = take(P * B * h->dims[L] * 4);
+  if (!h->small && (bf16 || !h->head)) h->off_Z = take(P * B * h->dims[L] * 4);
   h->off_loss = take(P * 4);
   h->off_err = take(16);
   // (a step that fits the static scratch without the pieces' partials has to fit it with them)
   if (fine_used && off > kStaticScratchBytes) return plan_layout(h, false);
   h->ws_step_bytes = off;
-  if (h->prec == HA_PREC_BF16 && h->S > 1) h->off_M = take((P / h->S) * h->ld * 4);
+  if (bf16 && !h->small && h->S > 1) h->off_M = take((P / h->S) * h->ld * 4);
   h->ws_bytes = off;
 }
 
@@ -1402,7 +1406,7 @@ int hier_avg_set_global_steps(hier_avg* h, int steps) {
 
 int hier_avg_set_batch(hier_avg* h, int B) {
   if (!h || B < 1 || B > h->B) return HA_EINVAL;
-  if (B < h->Bstep && h->bound && h->prec == HA_PREC_BF16) {
+  if (B < h->Bstep && h->bound && h->prec == HA_PREC_BF16 && !h->small) {
     // The bf16 path keeps Bn-row gradient tiles; rows from B on must add nothing to dW.
     DeviceScope scope(h->device);
     for (int l = 1; l <= h->L; ++l)

@@ -74,6 +74,25 @@ def test_layout_and_workspace(lib):
         lib.hier_avg_destroy(h)
 
 
+# The workspace holds what the handle's kernels read and no more: whole steps of a small net keep
+# theirs in shared memory, the fp32 path reads its first layer's rows from X, and the kernel of a
+# last layer of up to 16 classes writes neither its logits nor their gradient.
+@pytest.mark.parametrize("kw,most", [
+    (dict(P=6, S=3, B=20, dims=(264, 136, 200, 13), prec=1), 0),
+    (dict(P=4, S=2, B=7, dims=(100, 37, 10), prec=0), 0),
+    (dict(P=64, S=8, B=64, dims=(3072, 10), prec=0), 0),
+    (dict(P=16, S=4, B=32, dims=(3072, 512, 10), prec=0), 2 * 16 * 32 * 512 * 4),        # H_1, dZ_1
+    (dict(P=24, S=4, B=64, dims=(784, 512, 33), prec=0), 24 * 64 * (2 * 512 + 2 * 33) * 4),
+])
+def test_workspace_holds_what_is_read(lib, kw, most):
+    rc, h = _create(lib, **kw)
+    assert rc == 0
+    wb = ctypes.c_int64()
+    assert lib.hier_avg_workspace_bytes(h, ctypes.byref(wb)) == 0
+    lib.hier_avg_destroy(h)
+    assert most < wb.value <= most + 4 * kw["P"] + 8192             # losses, error word, alignment
+
+
 # Where the backward of few long tiles goes in pieces, the workspace holds the pieces' partials
 # (P tiles of 256 inputs in ceil(chunks / 4) pieces of 128 x Bn floats): from 17 chunks of 64
 # outputs on up to 32 samples, from 24 up to 48, from 32 up to 64.

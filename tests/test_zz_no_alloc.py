@@ -57,7 +57,16 @@ def _static_matches_bound(lib, w):
         assert lib.hier_avg_get_step(st.h, ctypes.byref(t)) == 0 and t.value == step + 1
 
 
-@pytest.mark.parametrize("w", [SMALL_BF16, configs.MLP512_P16, configs.SOFTMAX_P4],
+# Whole steps of a small net in one launch, in both precisions: nothing of a step is in the array
+# but the losses, and there are no tensor maps.  And an fp32 net past them, whose first layer has
+# no buffer.
+ONE_LAUNCH_BF16 = SMALL_BF16.replace(name="one_launch_bf16", P=6, S=3, dims=(264, 136, 200, 13), B=20, N=50)
+ONE_LAUNCH_FP32 = SMALL_BF16.replace(name="one_launch_fp32", dims=(100, 37, 10), precision="fp32", B=7, N=40)
+TILES_FP32 = SMALL_BF16.replace(name="tiles_fp32", dims=(784, 256, 33), precision="fp32", B=32, N=64)
+
+
+@pytest.mark.parametrize("w", [SMALL_BF16, configs.MLP512_P16, configs.SOFTMAX_P4, ONE_LAUNCH_BF16,
+                               ONE_LAUNCH_FP32, TILES_FP32],
                          ids=lambda w: w.name)
 def test_static_step_matches_bound_step(lib, w):
     assert torch.cuda.is_available(), "GPU tests need CUDA"
@@ -70,6 +79,8 @@ def test_static_step_after_a_larger_configuration(lib):
     assert torch.cuda.is_available(), "GPU tests need CUDA"
     _static_matches_bound(lib, LARGER_BF16)
     _static_matches_bound(lib, SMALL_BF16)
+    _static_matches_bound(lib, ONE_LAUNCH_BF16)
+    _static_matches_bound(lib, TILES_FP32)
 
 
 def test_static_step_rejects_large_configurations(lib):
