@@ -789,6 +789,58 @@ def test_backward_in_segment_pieces(w):
     test_literal_sequence_equals_round(w)
 
 
+# The pieces' partials are the sums that a whole tile adds in the same order.  12 learners of this
+# net have room for a static step's scratch only without them (a plan of whole tiles), 11 with
+# them; learners are independent until they are averaged and nothing else of the plan depends on
+# their number here, so the steps of the first 11 have to give the same bits.
+def test_backward_in_segment_pieces_gives_the_bits_of_whole_tiles():
+    dims = (13056, 128, 3072, 10)
+    whole = _head(dims, 12, 1, 64, 128)
+    partials = 12 * 128 * 64 * 4                                  # of one learner: 12 pieces
+    ha = {}
+    X, y = learner_data(whole)
+    layers = perturbed_layers(whole, 0.01, seed=7)
+    for P in (11, 12):
+        w = whole.replace(P=P)
+        ha[P] = HierAvg(P, 1, w.K1, w.K2, w.lr, w.B, dims, w.precision)
+        ha[P].bind(ha[P].pack(layers[:P]), X[:P].contiguous().cuda(), y[:P].contiguous().cuda())
+        for _ in range(2):
+            ha[P].step()
+        ha[P].check()
+    assert ha[12].workspace_bytes <= 32 << 20 < ha[12].workspace_bytes + 12 * partials
+    per_learner = ha[12].workspace_bytes / 12
+    assert ha[11].workspace_bytes > 11 * (per_learner + 0.9 * partials)
+    assert torch.equal(ha[11].params.view(torch.int32), ha[12].params[:11].view(torch.int32))
+    assert torch.equal(ha[11].losses(), ha[12].losses()[:11])
+
+
+# An fp32 data set may start anywhere (bind asks for 16 bytes in bf16 only): where the widths are
+# multiples of four, 4-byte copies of its rows meet 16-byte copies of the weights.  Which copies
+# move the operands changes no sum: the bits of the aligned data set.  A small net, one layer
+# (several steps per launch), and tiles with a last layer's kernel of their own and without.
+@pytest.mark.parametrize("w", [_fp32((100, 37, 10), 4, 2, 7), _fp32((3072, 10), 2, 2, 20),
+                               _fp32((784, 512, 10), 2, 1, 33), _fp32((260, 132, 300), 2, 2, 65)],
+                         ids=lambda w: w.name)
+@pytest.mark.parametrize("offset", [1, 2])
+def test_fp32_rows_off_16_bytes(w, offset):
+    X, y = learner_data(w)
+    layers = perturbed_layers(w, 0.01, seed=5)
+    buf = torch.empty(X.numel() + offset, dtype=torch.float32, device="cuda")
+    shifted = buf[offset:].view(X.shape)
+    shifted.copy_(X)
+    assert shifted.data_ptr() % 16 != 0
+    runs = []
+    for rows in (X.cuda(), shifted):
+        ha = HierAvg(w.P, w.S, w.K1, w.K2, w.lr, w.B, w.dims, w.precision)
+        ha.bind(ha.pack(layers), rows, y.cuda())
+        ha.round()
+        ha.step()
+        ha.check()
+        runs.append(ha)
+    assert torch.equal(runs[0].params.view(torch.int32), runs[1].params.view(torch.int32))
+    assert torch.equal(runs[0].losses(), runs[1].losses())
+
+
 # The cross-entropy over a cluster: fewer samples than its CTAs, a last CTA with fewer than
 # the others, more samples than threads, just past and just below the logits from which on it is
 # spread (12288), class slices of one partial tile and of more than one tile of 128 with an odd rest.
