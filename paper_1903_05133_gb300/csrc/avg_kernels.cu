@@ -465,7 +465,7 @@ int ilog2_exact(int64_t n) {
 
 // Fewer columns than about two waves of one-thread-per-column CTAs: split each column's
 // rows between two threads.
-constexpr int64_t kSplitCols = 2 * 152 * 8 * 256;
+constexpr int64_t kSplitCols = 2 * kSms * 8 * 256;
 bool split_rows(int64_t cols_v, int64_t groups) { return cols_v * groups <= kSplitCols; }
 
 // Grid of the power-of-two kernels: `per` quads per CTA, and a CTA for the columns after them.
@@ -537,7 +537,8 @@ void launch_lg(const float4* src, int64_t src_ld_v, float4* w, int64_t ld_v, int
     }
   }
   launch_pdl(tail != 0 ? k_local_global_pow2<LOGQ, LOGS, LOGG, kTail> : k_local_global_pow2<LOGQ, LOGS, LOGG, false>,
-             pow2_grid(cols_v, kThreads, tail, 1), dim3(kThreads), 0, s, false, 1, src, src_ld_v, w, ld_v, cols_v, tail);
+             pow2_grid(cols_v, kThreads, tail, 1), dim3(kThreads), 0, s, false, 1, src, src_ld_v, w, ld_v, cols_v,
+             tail);
 }
 
 template <int LOGQ, int LOGS>
@@ -591,7 +592,7 @@ void launch_mean_any(const float* src, int64_t ld, int64_t cols, int n, int64_t 
 }
 
 // Four columns per thread while that gives every SM two CTAs.
-bool spread_wide(int64_t cols, int64_t groups) { return cols * groups >= 2 * 152 * 1024; }
+bool spread_wide(int64_t cols, int64_t groups) { return cols * groups >= 2 * kSms * 1024; }
 
 template <bool kTo>
 void mean_any_dispatch(bool vec, const float* src, int64_t ld, int64_t cols, int n, int64_t groups,

@@ -24,7 +24,7 @@ using ha::TcBwdArgs;
 using ha::TcFwdArgs;
 
 constexpr int64_t kAlign = 1024;
-constexpr int64_t kTargetCtas = 152;   // persistent kernels: one CTA per SM of a GB300
+constexpr int64_t kTargetCtas = ha::kSms;   // persistent kernels: one CTA per SM
 constexpr int64_t kPieceChunks = 48;   // chunks per piece of a split tile (forward, backward)
 constexpr int64_t kFineChunks = 4;     // ... of a backward tile where few tiles leave SMs idle
 constexpr int64_t kStaticScratchBytes = int64_t(32) << 20;   // 32 MiB: step_static's scratch
@@ -242,8 +242,11 @@ void plan_layout(hier_avg* h, bool fine = true) {
   // Last layers of up to 16 classes run as one kernel.  In bf16, where the width is no multiple
   // of 64, that replaces the tensor-core forward and backward with their partly filled tiles:
   // 264-136-200-13 (P = 6, B = 20) 55 -> 43 us per step, one-layer 784-10 (P = 24, B = 64)
-  // 43 -> 15 us.  Wide layers after hidden ones keep the tensor-core kernels, whose tiles
-  // are nearly full there (2512 -> 10 behind 3072-512, P = 4: 1.6 % of the step).
+  // 43 -> 15 us.  Behind hidden layers widths over 1024 keep the tensor-core kernels all the same,
+  // not for speed (784-512-2008-10, P = 2 to 32: rounds in 0.77 to 0.95 of their time with this
+  // kernel; 3080 0.70 to 1.04): their long runs part with every change of rounding
+  // (3072-512-2512-10, 32 steps: either kernel's parameters 0.04 to 0.09 from 64-bit ones, 0.07
+  // from each other's), so results in use stay as they were.
   h->head = bf16 ? (wl % 64 == 0 || L == 1 || wl <= 1024) &&
                        ha::head_supported(h->dims[L], wl, static_cast<int>(B), h->P)
                  : ha::head32_supported(h->dims[L], wl, static_cast<int>(B));
@@ -258,7 +261,7 @@ void plan_layout(hier_avg* h, bool fine = true) {
     for (int l = 0; l < L; ++l) h->off_H[l] = take(P * h->Bn * h->pitch[l] * 2);
     for (int l = 1; l <= L; ++l) h->off_dZ[l] = take(P * h->Bn * h->pitch[l] * 2);
     // Stream-K plans of the forward and backward GEMMs: at most one persistent CTA
-    // per SM of a GB300 (152).  They depend on the shapes only, so the summation
+    // per SM of a GB300.  They depend on the shapes only, so the summation
     // order of split tiles is the same on every GPU.  Forward tile = 128 outputs x
     // 64-input chunks; backward tile = 128 inputs x 64-output chunks.
     h->fwd_group = h->S > 1 ? ha::tc_forward_group_size(h->S, h->Bn) : 1;
@@ -875,7 +878,7 @@ int do_step(hier_avg* h, bool h1_ready = false, bool fuse_next = false, bool* fu
         continue;
       }
       // The first layer's backward (no dX) runs the update-only kernel: independent
-      // runs of 8 chunks, claimed dynamically (measured faster than the backward
+      // runs of up to 8 chunks, claimed dynamically (measured faster than the backward
       // kernel's items for short layers too: 3072-512-10 round 0.859 -> 0.850 ms).
       // Grouped (q > 1): W_l read per learner, its group sums written to row g*q of the
       // W_l region, g < P / q.  A layer with dX first runs the backward without update

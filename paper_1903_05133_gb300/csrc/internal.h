@@ -9,6 +9,8 @@
 
 namespace ha {
 
+constexpr int kSms = 152;   // of a GB300
+
 // Launch through cudaLaunchKernelEx with programmatic stream serialization (the
 // kernel calls grid_dep_wait() before its first global access), optionally
 // cooperative (all CTAs resident at once) or as clusters of cluster_x CTAs.

@@ -111,8 +111,9 @@ struct WRows {
 // ------------------------------------------------------------------ forward and dX tiles
 // Both contract a [samples x K] operand (H, or dZ) with the weights into a tile of BM
 // samples x 64 columns.  The eight warps of a CTA split the reduction, not the tile: each
-// warp holds the whole tile (BM = 64: half of its samples) in registers, 8 columns by up
-// to 8 samples per thread, and takes an eighth of every 64-wide chunk of K, so that a
+// warp holds the whole tile (BM = 64: half of its samples) in registers (8 columns by up
+// to 8 samples per thread; from 32 samples on a few words of them spill at the 128 registers
+// that two CTAs per SM leave), and takes an eighth of every 64-wide chunk of K, so that a
 // chunk's 16-byte shared-memory reads feed 16 FFMAs each (half of the shared-memory
 // bandwidth at the FFMA rate).  With few tiles a cluster of up to 8 CTAs shares a tile's
 // chunks.  The partials meet in shared memory and then through distributed shared memory,
@@ -127,7 +128,6 @@ constexpr int kKC = 64;                 // reduction chunk
 constexpr int kKP = kKC + 4;            // row pitch: consecutive rows on distinct bank groups
 constexpr int kRP = kBN + 8;            // row pitch of the partials
 constexpr int kStages = 3;
-constexpr int kSms = 152;               // of a GB300
 
 __host__ __device__ constexpr int tile_stage_floats(int BM) { return (BM + kBN) * kKP; }
 __host__ __device__ constexpr int tile_smem(int BM) { return kStages * tile_stage_floats(BM) * 4; }
@@ -338,11 +338,12 @@ struct DwArgs {
   float* bias;
   int64_t ld;
   int in, out, B;
-  int vec_z, vec_h;            // 16-byte copies of dZ rows / of H and W rows
+  int vec_z;                   // 16-byte copies of dZ rows
   float lr;
 };
 
-template <bool kVec>           // a.vec_h: thread columns 4 lx .. 4 lx + 3 (+ 32), else lx + 8 n
+// kVec (16-byte copies of H and W rows): thread columns 4 lx .. 4 lx + 3 (+ 32), else lx + 8 n.
+template <bool kVec>
 __global__ void __launch_bounds__(kDwThreads, 3) k_dw_f32(const DwArgs a) {
   extern __shared__ __align__(16) float sm[];
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31, ly = lane_y(lane), lx = lane_x(lane);

@@ -8,12 +8,11 @@ namespace {
 using namespace head;
 
 // Features per CTA (a multiple of 64) for P learners: 8 CTAs per learner (slices of at
-// least 64) while all P clusters fit in one wave of the GPU's 152 SMs, else 4 (at least
+// least 64) while all P clusters fit in one wave of the GPU's SMs, else 4 (at least
 // 128; more clusters of 8 than fit at once measured slower), or 8 where 4 would need
 // slices over 512.
-constexpr int kHeadWave = 152;
 __host__ __device__ inline int head_slice(int in, int P) {
-  const bool wide = P * kHeadClusterMax <= kHeadWave;
+  const bool wide = P * kHeadClusterMax <= kSms;
   const int per = wide ? kHeadClusterMax : kHeadClusterPref;
   int f = ((in + per - 1) / per + 63) / 64 * 64;
   if (f > 512) f = ((in + kHeadClusterMax - 1) / kHeadClusterMax + 63) / 64 * 64;

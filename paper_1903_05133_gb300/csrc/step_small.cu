@@ -98,9 +98,9 @@ struct Div {
   __device__ __forceinline__ int operator()(int i) const { return d == 1 ? i : static_cast<int>(__umulhi(i, m)); }
 };
 
-// Partial products z[b][n] = sum_f h[b][f] w[n][f] of a slice: 4 samples (b, b + nb, ...) x 4 outputs
-// (n, n + no, ...), so that neighbouring lanes' rows fall on distinct banks, per KS neighbouring lanes, which take every KS-th quad of features and
-// then share out the 16 sums.
+// Partial products z[b][n] = sum_f h[b][f] w[n][f] of a slice: 4 samples (b, b + nb, ...) x 4
+// outputs (n, n + no, ...), so that neighbouring lanes' rows fall on distinct banks, per KS
+// neighbouring lanes, which take every KS-th quad of features and then share out the 16 sums.
 template <int KS>
 __device__ __forceinline__ void forward_slice(const float* h, const float* w, float* z, int F, int p, int op,
                                               int nb, int out, int t) {
@@ -365,9 +365,9 @@ __global__ void __launch_bounds__(kT, 2) k_small(const SmallArgs a) {
       const Div dq(q4);
       float* own = sm + o.own[l & 1];
       if (l > 0) {
-        // dZ_l of the own neurons: tiles of 4 samples (b, b + nb, ...) x 4
-        // neurons, the sum over the outputs
-        // split over ng groups of threads whose partials meet in the free z buffer
+        // dZ_l of the own neurons: tiles of 4 samples (b, b + nb, ...) x 4 neurons, the sum
+        // over the outputs split over ng groups of threads whose partials meet in the free z
+        // buffer
         const float* w = sm + o.wq[l];
         float* part = sm + o.z[ph];
         const int tiles = nb * q4;
@@ -487,19 +487,21 @@ __global__ void __launch_bounds__(kT, 2) k_small(const SmallArgs a) {
 
 // Nets that take these steps.  One wave of clusters: 15 of one CTA per SM, 19 where two fit an
 // SM (784-32-10 bf16, B = 64, a round of 8 steps: P = 16 366 -> 182 us, P = 64 209 -> 466).  Up
-// to 2 M multiply-adds per learner and forward, where the products of eight SMs begin to
-// outweigh the launches saved (784-40-10 bf16, P = 2, B = 64, just below: 213 -> 148 us;
-// 264-136-200-13, P = 6, B = 20, 1.3 M: 145 -> 82 us for 4 steps; fp32 100-37-10, P = 4, B = 7:
-// 49 -> 37 us; 512-96-80-10, P = 2, B = 32, 1.8 M, 8 steps: 271 -> 151 us).  One layer of up to
-// 16 classes stays with the head kernels (784-10 bf16, P = 16, B = 64, 28 steps: 308 against
-// 388 us here).
-constexpr int kSmallSms = 152;           // of a GB300
+// to 2 M multiply-adds per learner and forward.  Time here over that of the kernels per layer,
+// rounds of 8 steps | loops of 4 single steps: 0.7 to 1.4 M, P = 2 0.5-0.9 | 0.55-1.0, P = 16 0.45-1.0 |
+// 0.5-1.15; 2 to 2.8 M, P = 2 0.53-1.0 | 0.6-1.1; 4 M, P = 2 0.6-1.0 | 0.66-1.14, so past the line fewer
+// and fewer nets gain, and single steps of some lose.  (784-40-10 bf16, P = 2, B = 64, just below
+// it: 213 -> 148 us; 264-136-200-13, P = 6, B = 20, 1.3 M: 145 -> 82 us for 4 steps; fp32 100-37-10,
+// P = 4, B = 7: 49 -> 37 us; 512-96-80-10, P = 2, B = 32, 1.8 M, 8 steps: 271 -> 151 us; two of
+// 216 lose, single steps of fp32 784-128-10 and 1024-64-10, P = 16, B = 16: loops 74 -> 85 and 65 ->
+// 69 us, their rounds 151 -> 141 and 132 -> 114.)  One layer of up to 16 classes stays with the head
+// kernels (784-10 bf16, P = 16, B = 64, 28 steps: 308 against 388 us here).
 constexpr int kSmallClusters = 15;       // of eight CTAs that fill an SM each
 constexpr int kSmallSmemHalf = 112 * 1024;
 constexpr int64_t kSmallWork = int64_t(1) << 21;
 
 bool small_supported(const int* dims, int L, int B, int P, bool bf16) {
-  if (L > kSmallLayers || dims[L] > kSmallC || B > 64 || P * kR > kSmallSms) return false;
+  if (L > kSmallLayers || dims[L] > kSmallC || B > 64 || P * kR > kSms) return false;
   int64_t w = 0;
   for (int l = 0; l < L; ++l) w += static_cast<int64_t>(dims[l]) * dims[l + 1];
   if (w * B > kSmallWork) return false;

@@ -1674,7 +1674,7 @@ __global__ void __launch_bounds__(kBxThreads, 1)
 // for Q = 4), so that only this group sum is stored, to row q of the group-sum buffer
 // (store map) instead of Q learner rows.  The local average finishes the tree from
 // the group sums: the bits of the literal update and average.
-constexpr int kRun = 8;                 // chunks per work item
+constexpr int kRun = 8;                 // chunks per work item at most
 __host__ __device__ constexpr int upd_smem(int Bn) { return bwd_smem(Bn) + 512; }
 static_assert(upd_smem(64) <= kBwdSmemMax && upd_smem(48) <= kBwdSmemMax &&
                   upd_smem(32) <= kBwdSmemMax && upd_smem(16) <= kBwdSmemMax,
@@ -2705,7 +2705,6 @@ __global__ void __launch_bounds__(kXentThreads, 1) k_xent_bf16(const float* __re
 // 286 -> 265 us).  xent_spread says where it is the faster one.
 constexpr int kXentcThreads = 256, kXentRanks = 8, kXentTile = 128;
 constexpr int kXentSpread = 12288;               // logits per learner
-constexpr int kXentSms = 152;                    // of a GB300
 __global__ void __launch_bounds__(kXentcThreads) k_xent_bf16_cluster(const float* __restrict__ Z,
                                                            const int32_t* __restrict__ y,
                                                            int64_t N, int64_t row0, int B, int Bn,
@@ -2949,9 +2948,9 @@ cudaError_t launch_gather_bf16(const __nv_bfloat16* X, int64_t N, int d0, int B,
 // 56.7 | 47.1, 2000 104 | 132).
 static bool xent_spread(int64_t P, int64_t B, int64_t C) {
   if (B * C < kXentSpread) return false;
-  const int64_t waves = (P * ((C + kXentThreads - 1) / kXentThreads) + kXentSms - 1) / kXentSms;
+  const int64_t waves = (P * ((C + kXentThreads - 1) / kXentThreads) + kSms - 1) / kSms;
   if (waves == 1) return P <= 64 && C * std::max<int64_t>(P, 32) <= 1536 * B;
-  return kXentSms * waves >= 3 * P || (B >= 48 && 5 * kXentSms * waves >= 9 * P);
+  return kSms * waves >= 3 * P || (B >= 48 && 5 * kSms * waves >= 9 * P);
 }
 
 cudaError_t launch_xent_bf16(const float* Z, const int32_t* y, int64_t N, int64_t row0, int B,

@@ -284,8 +284,8 @@ def test_full_run_against_oracle(w):
 # per cluster); Q = 2 with S = 6 (three per cluster: the generic tree) and a ragged
 # 200-input layer; Q = 4 with S = 12 and K1 = 1 (every step both reads the cluster
 # means and writes group sums); Q = 2 because the batch is 64.
-# (Nets of these sizes run whole steps in one launch; test_group_sums_past_small_nets repeats
-# the cases on wider ones.)
+# (GROUP_S6 and GROUP_SP are small enough for whole steps in one launch, which store no group
+# sums; test_group_sums_past_small_nets has them, and the others, on wider nets.)
 GROUP_S8 = configs.Workload("mlp_bf16_group4_S8", P=16, S=8, K1=2, K2=3, rounds=1,
                             dims=(256, 192, 10), precision="bf16", N=128, B=32, lr=0.05,
                             sigma_mu=0.1, init="he")
@@ -675,7 +675,8 @@ def test_resume_from_saved_step():
 # sample missing or too many; widths that are no multiple of 4 (4-byte copies) or end inside
 # a 64-wide chunk; a reduction split over a cluster of 8 (one learner, 2048 inputs); the
 # small last layer at its limits (16 classes, 64 samples, slices of 64 features, one odd
-# slice) and just past them (17 classes, 65 samples, more than 8 x 1024 features).
+# slice) and just past them (17 classes, 65 samples, more than 8 x 1024 features).  (The smaller
+# of these nets run whole steps in one launch; the last three are past that.)
 def _fp32(dims, P, S, B, **kw):
     return configs.Workload("fp32_" + "-".join(map(str, dims)) + f"_P{P}_B{B}", P=P, S=S, K1=kw.get("K1", 2),
                             K2=2, rounds=1, dims=dims, precision="fp32", N=kw.get("N", 3 * B + 1), B=B,
@@ -686,7 +687,8 @@ FP32_CASES = [_fp32((64, 64, 17), 4, 2, 8), _fp32((130, 65, 40), 3, 1, 9), _fp32
               _fp32((100, 36, 10), 2, 1, 65), _fp32((2048, 64, 10), 1, 1, 32), _fp32((96, 72, 40), 2, 1, 130),
               _fp32((3072, 10), 2, 2, 64), _fp32((512, 16), 3, 1, 1), _fp32((37, 10), 4, 4, 17),
               _fp32((70, 5), 2, 2, 3), _fp32((8200, 10), 1, 1, 2), _fp32((516, 61, 16), 2, 1, 16),
-              _fp32((516, 61, 16), 2, 1, 31), _fp32((2048, 200, 10), 1, 1, 7)]
+              _fp32((516, 61, 16), 2, 1, 31), _fp32((2048, 200, 10), 1, 1, 7), _fp32((3000, 61, 16), 2, 1, 16),
+              _fp32((2048, 64, 17), 1, 1, 31), _fp32((8200, 10), 1, 1, 32)]
 
 
 @pytest.mark.parametrize("w", FP32_CASES, ids=lambda w: w.name)
@@ -743,7 +745,8 @@ def test_head_widths(w):
 # Whole steps of a small net in one launch, several between two averages: one to four layers,
 # widths below the eight slices of a learner and of odd length, 1 to 32 classes, batches of 1
 # to 64 that wrap around the data set (more than once in one launch), a last block shorter
-# than K1, odd clusters.
+# than K1, odd clusters, and 16 learners or more, two CTAs to an SM (1000-120-8 is just too large
+# for that and takes the kernels per layer).
 def _small(dims, precision, P, S, B, K1, N):
     return configs.Workload(f"small_{precision}_" + "-".join(map(str, dims)) + f"_P{P}_B{B}", P=P, S=S, K1=K1,
                             K2=2, rounds=1, dims=dims, precision=precision, N=N, B=B, lr=0.05, sigma_mu=0.1,
@@ -754,7 +757,8 @@ SMALL_CASES = [_small((100, 37, 10), "fp32", 4, 2, 7, 2, 40), _small((5, 3, 2), 
                _small((33, 64, 65, 7, 32), "fp32", 6, 2, 33, 2, 50), _small((300, 31), "fp32", 1, 1, 64, 3, 100),
                _small((264, 136, 200, 13), "bf16", 6, 3, 20, 4, 50), _small((8, 8, 1), "bf16", 2, 2, 1, 2, 1),
                _small((784, 40, 10), "bf16", 15, 5, 64, 3, 192), _small((136, 104, 88, 72, 32), "bf16", 5, 5, 17, 2, 20),
-               _small((1024, 17), "bf16", 18, 6, 48, 5, 96), _small((1000, 120, 8), "bf16", 16, 4, 16, 2, 64)]
+               _small((1024, 17), "bf16", 18, 6, 48, 5, 96), _small((1000, 120, 8), "bf16", 16, 4, 16, 2, 64),
+               _small((520, 72, 8), "bf16", 16, 4, 16, 2, 64)]
 
 
 @pytest.mark.parametrize("w", SMALL_CASES, ids=lambda w: w.name)
