@@ -724,7 +724,7 @@ def test_fp32_steps_in_one_launch(w, G):
 # features, half an MMA step), a width over 4 and over 8 CTAs whose last slice ends on an
 # odd multiple of 8, one class and 16, a one-layer model whose batches wrap, and a wide
 # one; over 1024 features behind a hidden layer, or 40 classes, stay with the cross-entropy in
-# the forward's epilogue.
+# the forward's epilogue.  The last two have 464 and 512 CTAs, four to an SM.
 def _head(dims, P, S, B, N):
     return configs.Workload("head_" + "-".join(map(str, dims)) + f"_P{P}_B{B}", P=P, S=S, K1=2, K2=2, rounds=1,
                             dims=dims, precision="bf16", N=N, B=B, lr=0.05, sigma_mu=0.1, init="he")
@@ -733,7 +733,7 @@ def _head(dims, P, S, B, N):
 HEAD_CASES = [_head((4096, 8, 10), 4, 2, 64, 256), _head((600, 200, 13), 6, 3, 20, 50),
               _head((128, 1000, 16), 24, 4, 33, 132), _head((4096, 520, 1), 2, 1, 1, 4),
               _head((3336, 10), 4, 4, 64, 90), _head((4104, 16), 2, 2, 64, 256), _head((64, 1032, 16), 2, 2, 64, 256),
-              _head((264, 200, 40), 6, 3, 20, 50)]
+              _head((264, 200, 40), 6, 3, 20, 50), _head((3072, 10), 58, 2, 16, 40), _head((64, 512, 13), 128, 4, 20, 60)]
 
 
 @pytest.mark.parametrize("w", HEAD_CASES, ids=lambda w: w.name)
